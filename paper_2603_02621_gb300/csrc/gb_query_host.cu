@@ -20,30 +20,52 @@ int gb_query_batch(gb_ctx* ctx, const uint64_t* n, uint32_t count, uint32_t P, u
     if (!n_dev)
         for (uint32_t i = 0; i < count; ++i)
             if ((n[i] & 1) || n[i] < 4 || n[i] >= (1ull << 63)) return fail(GB_EINVAL, "n must be even, 4 <= n < 2^63");
+    // host arrays go through pinned staging, one transfer each way (a single n
+    // as a kernel argument); device ones are used in place, with a count of
+    // the invalid n (host n were checked above)
+    constexpr uint32_t kStaged = 1u << 16;            // larger batches are copied as they are
+    const bool stage = count <= kStaged;
     int rc;
-    if ((!n_dev && (rc = ctx->qn.ensure((size_t)count * 8))) || (rc = ctx->qout.ensure((size_t)count * 4 + 16)))
+    if ((!n_dev && count > 1 && (rc = ctx->qn.ensure((size_t)count * 8))) ||
+        (rc = ctx->qout.ensure((size_t)count * 4 + 16)) ||
+        (stage && (rc = ctx->hstage.ensure((size_t)count * 12 + 16))))
         return rc;
-    const uint64_t* d_n = n;
-    if (!n_dev) {
-        GB_CUDA(ctx->copy(ctx->qn.p, n, (size_t)count * 8, cudaMemcpyHostToDevice, s));
-        d_n = ctx->qn.as<uint64_t>();
-    }
-    unsigned int* bad = reinterpret_cast<unsigned int*>(static_cast<unsigned char*>(ctx->qout.p) + (size_t)count * 4);
-    GB_CUDA(cudaMemsetAsync(bad, 0, 4, s));
+    unsigned char* const h_n = static_cast<unsigned char*>(ctx->hstage.p);
+    uint32_t* const h_out = reinterpret_cast<uint32_t*>(h_n + (size_t)count * 8);   // out, then the invalid count
     gb::QueryArgs qa{};
-    qa.n = d_n;
+    qa.n = n;
+    if (!n_dev) {
+        qa.n = ctx->qn.as<uint64_t>();
+        if (count == 1) {
+            qa.n = nullptr;
+            qa.n_inline = n[0];
+        } else {
+            if (stage) std::memcpy(h_n, n, (size_t)count * 8);
+            GB_CUDA(ctx->copy(ctx->qn.p, stage ? (const void*)h_n : n, (size_t)count * 8, cudaMemcpyHostToDevice, s));
+        }
+    }
+    uint32_t* const d_out = ctx->qout.as<uint32_t>();
+    qa.bad = n_dev ? d_out + count : nullptr;
+    if (n_dev) GB_CUDA(cudaMemsetAsync(qa.bad, 0, 4, s));
     qa.count = count;
     qa.primes = ctx->base->primes.as<uint32_t>();
     qa.recip = ctx->base->recip.as<uint64_t>();
     qa.n_filter = (uint32_t)(ctx->pi(gb::query_filter_max()) - 1);
     qa.K = (uint32_t)(ctx->pi(Pq) - 1);
-    qa.out = out_dev ? p_min : ctx->qout.as<uint32_t>();
-    qa.bad = bad;
+    qa.out = out_dev ? p_min : d_out;
     GB_LAUNCH(gb::launch_query(qa, s));
     unsigned int h_bad = 0;
-    GB_CUDA(ctx->copy(&h_bad, bad, 4, cudaMemcpyDeviceToHost, s));
-    if (!out_dev) GB_CUDA(ctx->copy(p_min, qa.out, (size_t)count * 4, cudaMemcpyDeviceToHost, s));
+    unsigned int* const bad_to = stage ? h_out + count : &h_bad;
+    if (!out_dev && n_dev && stage) {
+        GB_CUDA(ctx->copy(h_out, d_out, (size_t)count * 4 + 4, cudaMemcpyDeviceToHost, s));
+    } else {
+        if (n_dev) GB_CUDA(ctx->copy(bad_to, qa.bad, 4, cudaMemcpyDeviceToHost, s));
+        if (!out_dev)
+            GB_CUDA(ctx->copy(stage ? h_out : p_min, d_out, (size_t)count * 4, cudaMemcpyDeviceToHost, s));
+    }
     GB_CUDA(cudaStreamSynchronize(s));
+    if (!out_dev && stage) std::memcpy(p_min, h_out, (size_t)count * 4);
+    if (n_dev && stage) h_bad = *bad_to;
     if (h_bad) return fail(GB_EINVAL, "n must be even, 4 <= n < 2^63 (device input)");
     return GB_OK;
 }
