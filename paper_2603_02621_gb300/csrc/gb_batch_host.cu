@@ -64,8 +64,8 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     std::vector<uint32_t> groups;
     uint32_t nblk = 0;
     if (np > nmid) {
-        const uint64_t chunk = ctx->large_chunk_bits;
-        uint64_t acc = 0;
+        const uint64_t chunk = std::min(ctx->large_chunk_bits, gb::kMaxPieceBits);
+        uint64_t acc = 0, q_bit = 0;                        // q_bit: the range's window in the batch buffer
         uint32_t most = 0;
         groups.push_back(0);
         for (uint32_t i = 0; i < count; ++i) {
@@ -81,10 +81,20 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
                     groups.push_back((uint32_t)pieces.size());
                     acc = 0;
                 }
-                pieces.push_back(gb::LargePiece{i, nl, b0, b1});
+                const int64_t b = Bi + 2 * (int64_t)b0;
+                const uint64_t nbelow = b > 0 ? ctx->pi(isqrt_u64((uint64_t)b)) : 0;
+                gb::LargePiece pc{};
+                pc.b = b;
+                pc.bit0 = q_bit + b0;
+                pc.span = (uint32_t)(b1 - b0);
+                pc.n_primes = nl;
+                pc.n_below = nbelow > nmid ? (uint32_t)(nbelow - nmid) : 0u;
+                pc.b_mod210 = (uint32_t)((b % 210 + 210) % 210);
+                pieces.push_back(pc);
                 acc += b1 - b0;
                 most = std::max(most, nl);
             }
+            q_bit += nb;
         }
         groups.push_back((uint32_t)pieces.size());
         for (size_t g = 0; g + 1 < groups.size(); ++g)
@@ -98,7 +108,8 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     if (n_large_items > 0xffffffffull) return fail(GB_EINVAL, "batch too large");
 
     // device buffers
-    const size_t desc_ranges = (size_t)count * sizeof(gb::BatchRange) + n_pieces * sizeof(gb::LargePiece);
+    const size_t desc_pieces = ((size_t)count * sizeof(gb::BatchRange) + 15) & ~size_t(15);    // (16-byte loads)
+    const size_t desc_ranges = desc_pieces + n_pieces * sizeof(gb::LargePiece);
     const size_t desc_bytes = desc_ranges + (size_t)(2 * n_sieve + 2 * n_cover + 2 * n_mid) * 4 +
                               (size_t)(n_groups + 1) * 4 + 64;
     const bool want_rows = hist && hist_stride;
@@ -117,7 +128,7 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     // cover items | piece groups | mid items | counts
     unsigned char* hs_p = static_cast<unsigned char*>(ctx->hstage.p);
     gb::BatchRange* hr = reinterpret_cast<gb::BatchRange*>(hs_p);
-    gb::LargePiece* hpc = reinterpret_cast<gb::LargePiece*>(hs_p + (size_t)count * sizeof(gb::BatchRange));
+    gb::LargePiece* hpc = reinterpret_cast<gb::LargePiece*>(hs_p + desc_pieces);
     std::memcpy(hpc, pieces.data(), n_pieces * sizeof(gb::LargePiece));
     uint32_t* s_range = reinterpret_cast<uint32_t*>(hs_p + desc_ranges);
     uint32_t* s_tile = s_range + n_sieve;
@@ -159,7 +170,7 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     const size_t used = reinterpret_cast<unsigned char*>(counts + 5) - hs_p;
     GB_CUDA(ctx->copy(dd, hs_p, used, cudaMemcpyHostToDevice, s));
     const gb::BatchRange* d_ranges = reinterpret_cast<const gb::BatchRange*>(dd);
-    const gb::LargePiece* d_pieces = reinterpret_cast<const gb::LargePiece*>(dd + (size_t)count * sizeof(gb::BatchRange));
+    const gb::LargePiece* d_pieces = reinterpret_cast<const gb::LargePiece*>(dd + desc_pieces);
     const uint32_t* d_s_range = reinterpret_cast<const uint32_t*>(dd + desc_ranges);
     const uint32_t* d_s_tile = d_s_range + n_sieve;
     const uint32_t* d_c_range = d_s_tile + n_sieve;
@@ -216,7 +227,6 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
         GB_LAUNCH(gb::launch_sieve_items(sa, (int)cfg.cta_threads, ls));
         {
             gb::LargeBatchArgs la{};
-            la.ranges = d_ranges;
             la.pieces = d_pieces;
             la.groups = d_groups;
             la.nblk = nblk;

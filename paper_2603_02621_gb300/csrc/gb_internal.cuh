@@ -92,11 +92,40 @@ __device__ __forceinline__ uint32_t neg_mod(int64_t b, uint32_t p, uint64_t m)
     return t ? p - t : 0u;
 }
 
+// The same for b > 0 and 5p < 2^32 in 32-bit words: the quotient is needed
+// mod 2^32 only, and of its four partial products the lowest and the carries
+// between the rest are dropped, which leaves it at most 4 below floor(b/p)
+// (2 from the reciprocal, 2 from the dropped fractions), so the remainder is
+// below 5p: 3 + 1 multiply-adds and 6 more instructions, against about 30 with
+// 64-bit products and compares.
+constexpr uint32_t kLowModMax = 858993459u;     // floor((2^32 - 1) / 5)
+__host__ __device__ __forceinline__ uint32_t mulhi_u32(uint32_t a, uint32_t b)
+{
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+}
+__host__ __device__ __forceinline__ uint32_t neg_mod_low(uint64_t b, uint32_t p, uint64_t m)
+{
+    const uint32_t bh = (uint32_t)(b >> 32), bl = (uint32_t)b, mh = (uint32_t)(m >> 32), ml = (uint32_t)m;
+    const uint32_t q = bh * mh + mulhi_u32(bh, ml) + mulhi_u32(bl, mh);
+    uint32_t r = bl - q * p;                                // < 5p
+    uint32_t s = r - 2 * p;                                 // (wraps above r when r < 2p)
+    r = s < r ? s : r;
+    s = r - 2 * p;
+    r = s < r ? s : r;                                      // < 2p
+    s = r - p;
+    r = s < r ? s : r;
+    return r ? p - r : 0u;
+}
+
 // Index i >= 0 of the first odd multiple of p in the odd-number sequence
 // b, b+2, b+4, ... (b odd): 2i = -b (mod p), i < p.
 __device__ __forceinline__ uint32_t first_odd_multiple(int64_t b, uint32_t p, uint64_t m)
 {
-    uint32_t r = neg_mod(b, p, m);
+    if (b > 0 && p <= kLowModMax) {
+        const uint32_t r = neg_mod_low((uint64_t)b, p, m);
+        return (r + ((r & 1u) ? p : 0u)) >> 1;
+    }
+    const uint32_t r = neg_mod(b, p, m);
     return (r & 1u) ? (uint32_t)(((uint64_t)r + p) >> 1) : (r >> 1);
 }
 
@@ -374,14 +403,18 @@ cudaError_t launch_mid_items(const MidItemsArgs& a, cudaStream_t s);
 // L2; a long window is cut into several pieces): items (group, block of 256
 // primes), group-major, from a device queue; a thread stops at the first
 // piece of its group that its prime does not reach
-// a run of one range's window bits, at most an L2-sized chunk
-struct LargePiece {
-    uint32_t range;
+// a run of one range's window bits, at most an L2-sized chunk; everything a
+// prime's start needs in three 16-byte words
+struct alignas(16) LargePiece {
+    int64_t  b;                 // number of the piece's first bit
+    uint64_t bit0;              // that bit in the batch buffer
+    uint32_t span;              // bits (<= 2^31)
     uint32_t n_primes;          // large primes with p^2 <= the piece's last number
-    uint64_t bit_lo, bit_hi;
+    uint32_t n_below;           // of these, the ones with p^2 <= b
+    uint32_t b_mod210;          // b mod 210, >= 0 also for b < 0
 };
+constexpr uint64_t kMaxPieceBits = 1ull << 31;
 struct LargeBatchArgs {
-    const BatchRange* ranges;
     const LargePiece* pieces;   // grouped; within a group by n_primes, descending
     const uint32_t* groups;     // device: first piece of each group, then the count
     uint32_t nblk;              // blocks of 256 primes per group (the most any piece needs)
@@ -461,16 +494,17 @@ struct PartitionArgs {
 cudaError_t launch_reverse_bits(const uint32_t* P, uint32_t* rev, uint64_t words, cudaStream_t s);
 cudaError_t launch_partitions(const PartitionArgs& a, cudaStream_t s);
 
-// Single-n queries (gb_query.cu): one CTA per n, p_min over primes[1..K]
+// Single-n queries (gb_query.cu): one warp per n, p_min over primes[1..K]
 struct QueryArgs {
-    const uint64_t* n;          // device: even n, 4 <= n < 2^63
+    const uint64_t* n;          // device: even n, 4 <= n < 2^63 (NULL: the one n_inline)
+    uint64_t n_inline;
     uint32_t count;
     const uint32_t* primes;     // [2, 3, 5, ...]
     const uint64_t* recip;
     uint32_t n_filter;          // pre-sieve primes primes[1..n_filter] (all odd primes <= query_filter_max())
     uint32_t K;                 // candidates primes[1..K] (p <= P)
     uint32_t* out;              // device: p_min, 0 if no p <= P
-    unsigned int* bad;          // device: count of invalid n (their out is 0)
+    unsigned int* bad;          // device, optional: count of invalid n (their out is 0)
 };
 cudaError_t launch_query(const QueryArgs& a, cudaStream_t s);
 uint32_t query_filter_max();

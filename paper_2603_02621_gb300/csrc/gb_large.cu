@@ -37,59 +37,13 @@
 // of chunks not yet visited is harmless, the strikes only clear composite
 // bits), and the event is counted.
 #include "gb_internal.cuh"
+#include "gb_wheel210.cuh"
 
 namespace gb {
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr uint32_t kWheelPos = 48;          // residues mod 210 coprime to 210
-
-constexpr bool coprime210(int r) { return r % 2 != 0 && r % 3 != 0 && r % 5 != 0 && r % 7 != 0; }
-
-struct Wheel210 {
-    uint8_t hgap[kWheelPos];    // half gap from wheel position w to w + 1 (position 47 -> 0: 209 -> 211)
-    uint8_t inv[210];           // p^-1 mod 210 for p coprime to 210 (0 elsewhere)
-    uint16_t next[210];         // odd r: position of the first coprime residue >= r | half the distance << 6
-};
-
-constexpr Wheel210 make_wheel210()
-{
-    Wheel210 t{};
-    int res[kWheelPos + 1] = {};
-    int n = 0;
-    for (int r = 1; r < 210; ++r)
-        if (coprime210(r)) res[n++] = r;
-    res[kWheelPos] = 211;                   // 1 + 210: the first residue of the next period
-    for (int w = 0; w < (int)kWheelPos; ++w) t.hgap[w] = (uint8_t)((res[w + 1] - res[w]) / 2);
-    for (int p = 1; p < 210; ++p)
-        if (coprime210(p))
-            for (int u = 1; u < 210; ++u)
-                if (p * u % 210 == 1) t.inv[p] = (uint8_t)u;
-    for (int r = 1; r < 210; r += 2) {
-        int w = 0;
-        while (res[w] < r) ++w;             // res[48] = 211 >= every r
-        t.next[r] = (uint16_t)((w % (int)kWheelPos) | (((res[w] - r) / 2) << 6));
-    }
-    return t;
-}
-__constant__ Wheel210 kWheel210 = make_wheel210();
-
-// the wheel tables in shared memory (lanes read different entries)
-struct WheelShared {
-    uint8_t hgap[kWheelPos];
-    uint8_t inv[210];
-    uint16_t next[210];
-};
-__device__ __forceinline__ void load_wheel(WheelShared& ws)
-{
-    for (uint32_t t = threadIdx.x; t < 210; t += blockDim.x) {
-        ws.inv[t] = kWheel210.inv[t];
-        ws.next[t] = kWheel210.next[t];
-        if (t < kWheelPos) ws.hgap[t] = kWheel210.hgap[t];
-    }
-}
-
 // a sparse entry: p / 2 (p odd, < 2^31) << 34 | wheel position << 28 | offset in the chunk (< 2^28)
 __device__ __forceinline__ uint64_t make_entry(uint32_t p, uint32_t w, uint32_t o)
 {
@@ -184,10 +138,7 @@ __global__ void __launch_bounds__(kThreads) k_large_start(const BucketLargeArgs 
         if (k < n) {
             p = a.primes[k];
             const uint64_t i0 = first_odd_multiple(a.B, p, a.recip[k]);        // < p
-            // m0 = (B + 2 i0) / p is odd; its residue mod 210 from (B + 2 i0) mod 210
-            const uint32_t r = (a.B_mod210 + 2u * (uint32_t)(i0 % 105u)) % 210u;
-            const uint32_t mr = (r * (uint32_t)ws.inv[p % 210u]) % 210u;
-            const uint32_t nx = ws.next[mr];
+            const uint32_t nx = wheel_entry(ws, p, a.B_mod210, (uint32_t)i0);
             w = nx & 63u;
             const uint64_t i = i0 + (uint64_t)p * (nx >> 6);                 // < 5p
             if (k < a.n_dense) {
