@@ -21,9 +21,12 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     const uint32_t H = 64 * ((P1 + 1 - 4 + 63) / 64) + 4;     // first-pass halo
     const uint32_t hs = K1 + 1;                               // device histogram row
     const uint32_t T = cfg.tile_bits;
-    const uint32_t cw = 3840;                                 // block-cover CTA chunk (64-bit words)
     GB_CUDA(cudaSetDevice(cfg.device));
     cudaStream_t s = ctx->stream;
+
+    uint64_t n_words = 0;
+    for (uint32_t i = 0; i < count; ++i) n_words += hi[i] > lo[i] ? ((hi[i] - lo[i]) / 2 + 31) / 32 : 0;
+    const uint32_t cw = gb::cover_chunk_words(n_words, false);   // block-cover CTA chunk (32-bit words)
 
     // per-range windows and work items
     uint64_t qwords = 0, n_sieve = 0, n_cover = 0, hi_max = 0, last_max = 0;
@@ -35,7 +38,7 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
         const uint64_t qw = (n + 63) / 64 + H / 128 + 2;
         qwords += qw;
         n_sieve += (64 * qw + T - 1) / T;
-        n_cover += (((n + 31) / 32) + 2ull * cw - 1) / (2ull * cw);
+        n_cover += ((n + 31) / 32 + cw - 1) / cw;
         hi_max = std::max(hi_max, hi[i]);
         last_max = std::max(last_max, lo[i] - H + 1 + 2 * (64 * qw - 1));   // window's last number
     }
@@ -152,7 +155,7 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
             off += qw;
             const uint64_t tiles = (64 * qw + T - 1) / T;
             for (uint64_t t = 0; t < tiles; ++t) { s_range[si] = i; s_tile[si] = (uint32_t)t; ++si; }
-            const uint64_t chunks = (((n + 31) / 32) + 2ull * cw - 1) / (2ull * cw);
+            const uint64_t chunks = ((n + 31) / 32 + cw - 1) / cw;
             for (uint64_t c = 0; c < chunks; ++c) { c_range[ci] = i; c_chunk[ci] = (uint32_t)c; ++ci; }
             if (n_mid) {
                 const uint64_t slices = (64 * qw + gb::kMidSliceBits - 1) / gb::kMidSliceBits;

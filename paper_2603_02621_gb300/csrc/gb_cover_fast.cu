@@ -1,40 +1,57 @@
-// gb_cover_fast.cu -- two-phase form of the loop-inverted Goldbach cover.
+// gb_cover_fast.cu -- block form of the loop-inverted Goldbach cover.
 //
 // Same computation as the generic cover (gb_cover.cu): for p = 3, 5, 7, ... <= P
 // in ascending order, every even n whose partner n - p is prime and that no
 // smaller p covered gets p_min(n) = p (GoldbachGPU, arXiv 2603.02621, Sec.
 // 2.3.1-2.3.2, in the bitwise form of Sec. 4.3).  Only the schedule differs.
 //
-// Unrolled blocks.  Most n are covered by one of the first few dozen primes,
-// so primes are applied in blocks unrolled at compile time.  A lane owns one
-// 32-bit word of C (32 even n) at a time.  With the halo chosen so that
-// d_3 = (H - 4)/2 is a multiple of 32, the partner bits of word w for the
-// prime p start at bit 32(w + d_3/32) - (p-3)/2 of Q: the word offset and the
-// shift of every step are compile-time constants, and the few Q words a lane
-// needs sit in registers.  A step is then
+// Classes mod 3.  For half of the primes p the partner of an n not divisible by
+// 3 is a multiple of 3, and a step over a word of consecutive n works for two
+// n in three.  So the n are taken by their residue v mod 3, each class with its
+// own useful primes: for v = 0 all from 5 on, for v = 1 those = 2 (mod 3) and 3,
+// for v = 2 those = 1 (mod 3) and 3 (the partner 3 itself is p_min's only for
+// n = 6, set apart like n = 4 = 2 + 2).  A word of one class comes from three
+// places: a chunk of the window is cut into three streams of O words each, O not
+// a multiple of 3, and since 32 = 2 (mod 3) the bits of one residue sit at three
+// different phases in the words k, k + O and k + 2 O; an AND with the phase's
+// mask and an OR put them side by side into one word, at the bit positions they
+// had.  That is done once per chunk for the q of residue 1 and 2 (2 logic
+// operations per word; q divisible by 3 drop out), into shared memory.  A shift
+// by (p - 3)/2 bits then means the same in the merged words as in the window's,
+// so a step is what it was, over words of 32 n of one class, and only two thirds
+// of the steps are left.
+//
+// Steps.  With the halo chosen so that d_3 = (H - 4)/2 is a multiple of 32, the
+// partner bits of word w for the prime p start at bit 32(w + d_3/32) - (p-3)/2 of
+// Q: the word offset and the shift of every step are compile-time constants, and
+// the few words a lane needs sit in registers.  A step is then
 //     s = funnel-shift of two window registers,  C |= s,  cum_k += popc(C)
 // and the histogram follows from the cumulative counts:
 // #{n : p_min(n) = p_k} = cum_k - cum_{k-1} (three counts per register, added
-// by multiply-adds with the field weights).  Block 0 (L0 primes) runs on
-// every word of the CTA, three consecutive words per lane sharing one window;
-// the words it leaves open (about one in three after 48 primes near 1e10) go
-// to per-warp lists in shared memory, and blocks of 32 primes run on the open
-// words alone, each leaving a shorter list, so that every lane of every step
-// still works on an open word.  The prefix KA = L0 + 32 x (later blocks).
+// by multiply-adds with the field weights).  Block 0 (L0 useful primes) runs on
+// every word of the class, three consecutive words per lane sharing one window;
+// the words it leaves open (about one in four after 32 useful primes near 5e11)
+// go to per-warp lists in shared memory, and blocks of 16 run on the open words
+// alone, each leaving a shorter list.
 //
-// Probing.  The few n open after the last block (about 1 in 10^4 after 112
-// primes near 1e10)
-// are taken one at a time by a warp: lane t probes the bit of Q at j + d_k for
-// k = k0 + t, and the lowest set bit of the ballot is p_min.  An n still open
+// Probing.  The few n open after the last block, or in the last few words of a
+// list, are taken one at a time by a warp: lane t probes the bit of Q at j + d_k
+// for k = k0 + t, and the lowest set bit of the ballot is p_min.  An n still open
 // after K primes goes to the retry pass (or counts as unresolved).
 //
-// The largest p_min of a warp's words, with its smallest n, comes from the
-// probing when any n reached it.  Otherwise it lies in the last block that set
-// a bit (known from the histogram), and that block is run once more over its
-// input words, recording per word the last step that set a bit and the bits it
-// set.  A later block writes its output list above its input when there is
-// room, so that the input is still there for this re-run; when there is not,
-// the warp's words are re-run through every block up to that one.
+// The largest p_min, with its smallest n, of a warp's words of a class comes
+// from the probing when any n reached it: every n of the class covered by the
+// blocks has a smaller one.  Where a later block covers all that was open, its
+// input list is still there and is run once more, recording it; where block 0
+// does (a few words only), the words are, unless block 0's last prime is below
+// the chunk's maximum so far.
+//
+// Bound: the ALU pipe and the popcounts of block 0 (a step on three words is 8
+// ALU, 2 popcount and 3 multiply-add instructions).  2^32 n from 4 on, 2^33
+// near 5e11, 2^31 near 1e15 and 2^32 below 4e18 on a GB300: 1.69, 3.86, 1.26 and
+// 3.13 ms without the classes (48 or 64 primes over every word, blocks of 32),
+// 1.15, 2.64, 0.87 and 2.02 ms with them.
+#include <algorithm>
 #include <type_traits>
 #include <utility>
 
@@ -43,94 +60,120 @@
 
 namespace gb {
 
-// k-th odd prime (k = 0 -> 3), evaluated at compile time
-__host__ __device__ constexpr uint32_t odd_prime(int k)
+// cumulative counts are kept three per register (10-bit fields): a lane adds
+// at most 96 per round of three words and runs at most ten rounds, or at most
+// 32 per listed word and handles at most 30 of them (960 < 2^10)
+constexpr int kCumBits = 10;
+constexpr uint32_t kCumMask = (1u << kCumBits) - 1;
+constexpr uint32_t kMaxRounds = 10;
+
+// schedule: block 0 of L0 useful primes, then at most kMaxLater blocks of kLater
+constexpr int kLater = 16;
+constexpr int kMaxUseful = 128;
+constexpr int kMaxPrefix = 256;
+// a list this short is probed rather than run through another block (a block
+// costs about 150 warp instructions, an open n about 40; 2^33 n near 5e11: 2.66
+// ms with 1, 2.64 with 3, 2.71 with 8, 2.86 with 16)
+constexpr uint32_t kProbeWords = 3;
+
+// Threads per CTA, and rounds of merged words (96 per warp) per class and chunk.
+// Two CTAs of 512 per SM, each warp through one class after the other: their
+// sixteen warps are mostly in the same code (see block0_class).  A chunk has
+// fixed costs (the counts' flushes, the merging's ends, the last words' probing),
+// so it is as long as shared memory allows, five rounds (103 KB) -- 2^33 n near
+// 5e11 take 2.83 ms with four and 2.64 with five; 2.65 with 256 threads, four
+// CTAs and a barrier between the classes, 2.97 with 1024 -- unless the call is
+// too small to give every SM its chunks.
+constexpr int kCoverNT = 512, kFusedNT = 256;
+constexpr int kCoverCtas = 2;                               // per SM
+constexpr uint32_t kRounds = 5;
+constexpr uint32_t kFusedRounds = 3;                        // (the fused tile holds no more)
+static_assert(kRounds <= kMaxRounds, "10-bit counters");
+// words per chunk: three streams of 3 NT R - 1 words (not a multiple of 3)
+uint32_t cover_chunk_words(uint64_t words, bool fused)
 {
-    uint32_t c = 1;
-    int n = -1;
-    while (n < k) {
-        c += 2;
+    if (fused) return 3 * (3 * kFusedNT * kFusedRounds - 1);
+    const uint64_t round = 9ull * kCoverNT, slots = (uint64_t)kCoverCtas * device_sms();
+    const uint64_t r = std::min<uint64_t>(std::max<uint64_t>((words + round * slots - 1) / (round * slots), 1), kRounds);
+    return (uint32_t)(3 * (3 * kCoverNT * r - 1));
+}
+
+// useful primes of the classes: p[v][i], k[v][i] = its index among the odd primes
+struct ClassPrimes {
+    uint16_t p[3][kMaxUseful], k[3][kMaxUseful];
+};
+constexpr ClassPrimes make_class_primes()
+{
+    ClassPrimes t{};
+    int n[3] = {0, 0, 0};
+    int k = 0;
+    for (uint32_t c = 3; n[0] < kMaxUseful || n[1] < kMaxUseful || n[2] < kMaxUseful; c += 2) {
         bool prime = true;
         for (uint32_t d = 3; d * d <= c; d += 2)
             if (c % d == 0) { prime = false; break; }
-        if (prime) ++n;
+        if (!prime) continue;
+        for (uint32_t v = 0; v < 3; ++v)
+            if (c % 3 != v && n[v] < kMaxUseful) {
+                t.p[v][n[v]] = (uint16_t)c;
+                t.k[v][n[v]] = (uint16_t)k;
+                ++n[v];
+            }
+        ++k;
     }
-    return c;
+    return t;
 }
+constexpr ClassPrimes kClass = make_class_primes();
+__constant__ ClassPrimes kClassDev = make_class_primes();
 
-// cumulative counts are kept three per register (10-bit fields): a lane adds
-// at most 32 per word and handles at most 30 listed words (or 10 rounds of
-// three words) per CTA in a block (32 * 30 < 2^10)
-constexpr int kCumBits = 10;
-constexpr uint32_t kCumMask = (1u << kCumBits) - 1;
+// step I of class V: the prime's (p - 3)/2, the word offset of its partner bits
+// and the residue of the partners
+constexpr uint32_t use_e(int V, int I) { return (kClass.p[V][I] - 3u) / 2; }
+constexpr int use_c(int V, int I) { return (int)((use_e(V, I) + 31) / 32); }
+constexpr int use_rho(int V, int I) { return (V + 3 - kClass.p[V][I] % 3) % 3; }
+template <int V, int I>
+struct Step {
+    static constexpr int c = use_c(V, I), rho = use_rho(V, I);
+    static constexpr uint32_t sh = 32u * (uint32_t)use_c(V, I) - use_e(V, I);
+};
 
-// schedule: block 0 of L0 primes, then at most kMaxLater blocks of kLater
-constexpr int kLater = 32;
-constexpr int kMaxLater = 6;
-constexpr int kMaxPrefix = 64 + kLater * kMaxLater;
-
-// a warp's list holds every word it takes in block 0 (ten rounds of 96 words
-// at most: the 10-bit counters allow no more)
-__host__ __device__ constexpr uint32_t list_cap(uint32_t cta_words, int NW)
+// window of the steps [I0, I0 + L) of class V in the merged words of residue
+// rho: word offsets lo .. lo + n - 1 below the word's own
+constexpr int win_lo(int V, int I0, int L, int rho)
 {
-    return (2 * cta_words + 96 * NW - 1) / (96 * NW) * 96;
+    int lo = 1 << 20;
+    for (int i = I0; i < I0 + L; ++i)
+        if (use_rho(V, i) == rho && use_c(V, i) - 1 < lo) lo = use_c(V, i) - 1;
+    return lo < 0 || lo == 1 << 20 ? 0 : lo;
 }
-
-__host__ __device__ constexpr uint32_t step_e(int k) { return (odd_prime(k) - 3) / 2; }
-// window of a block of L primes from index K0: R[t] = Q32[base - C0 - t]
-// with C0 = the first step's word offset - 1
-__host__ __device__ constexpr int block_c0(int K0)
+constexpr int win_n(int V, int I0, int L, int rho)
 {
-    return K0 == 0 ? 0 : (int)((step_e(K0) + 31) / 32) - 1;
+    int hi = -1;
+    for (int i = I0; i < I0 + L; ++i)
+        if (use_rho(V, i) == rho && use_c(V, i) > hi) hi = use_c(V, i);
+    return hi < 0 ? 0 : hi - win_lo(V, I0, L, rho) + 1;
 }
-__host__ __device__ constexpr int block_regs(int K0, int L)
-{
-    return (int)((step_e(K0 + L - 1) + 31) / 32) - block_c0(K0) + 1;
-}
+template <int V, int I0, int L, int RHO>
+struct Win {
+    static constexpr int lo = win_lo(V, I0, L, RHO), n = win_n(V, I0, L, RHO);
+};
 
-template <int K, int K0, int NR>
-__device__ __forceinline__ uint32_t window_shift(const uint32_t (&R)[NR])
-{
-    constexpr uint32_t e = step_e(K);
-    constexpr int c = (int)((e + 31) / 32);
-    constexpr uint32_t sh = 32 * c - e;
-    constexpr int r = c - block_c0(K0);
-    static_assert(r >= 0 && r < NR, "window too small");
-    if constexpr (sh == 0) return R[r];
-    else return __funnelshift_r(R[r], R[r - 1], sh);
-}
+// bits b = phi (mod 3) of a word, phi in 0 .. 2
+__device__ __forceinline__ uint32_t phase_mask(uint32_t phi) { return 0x49249249u << phi; }
+__device__ __forceinline__ uint32_t mod3(uint32_t x) { return x % 3u; }
 
-template <int K, int K0, int NR, int KH>
-__device__ __forceinline__ void block_step(const uint32_t (&R)[NR], uint32_t& C, uint32_t (&cum)[KH],
-                                           const uint32_t (&wt)[3])
-{
-    C |= window_shift<K, K0, NR>(R);
-    constexpr int j = K - K0;
-    cum[j / 3] = __popc(C) * wt[j % 3] + cum[j / 3];
-}
-
-template <int K0, int NR, int KH, int... J>
-__device__ __forceinline__ void run_block(std::integer_sequence<int, J...>, const uint32_t (&R)[NR], uint32_t& C,
-                                          uint32_t (&cum)[KH], const uint32_t (&wt)[3])
-{
-    (block_step<K0 + J, K0, NR, KH>(R, C, cum, wt), ...);
-}
-
-// add one block's histogram to shist; kmax becomes the largest bin (prime
-// index + 1) the block added to, if any.  The lanes' cumulative counts are
-// summed over the warp by a transposed butterfly: two counts per register as
+// add one block's histogram to the class's bins, from the block's first on.  The lanes' cumulative counts
+// are summed over the warp by a transposed butterfly: two counts per register as
 // 16-bit fields (a lane's counts are at most 960, a warp's at most 30720), and
 // at each of five shuffle stages a lane keeps half of its registers and sends
 // the other half to its partner, so that lane l ends with the warp totals of
-// the counts 2l and 2l + 1 (L / 2 = 32 registers, padded from 24 for L = 48)
-// or, for L = 32, of the counts 2(l/2) and 2(l/2) + 1 (lanes l and l ^ 1
-// alike).  The bins are the differences of consecutive totals.
-template <int K0, int L, int KH>
-__device__ __forceinline__ void flush_block(const uint32_t (&cum)[KH], uint32_t init_pop, uint32_t* shist, int lane,
-                                            uint32_t& kmax)
+// the count pair l (L > 32: registers padded to 32), l / 2 (L > 16) or l / 4.
+// The bins are the differences of consecutive totals.
+template <int L, int KH>
+__device__ __forceinline__ void flush_block(const uint32_t (&cum)[KH], uint32_t init_pop, uint32_t* first_bin, int lane)
 {
     constexpr int NP = L / 2;                               // count pairs
-    constexpr int NR = NP <= 16 ? 16 : 32;                  // registers, a power of two
+    constexpr int NR = NP <= 8 ? 8 : NP <= 16 ? 16 : 32;    // registers, a power of two
+    constexpr int SH = NR == 8 ? 2 : NR == 16 ? 1 : 0;      // lane >> SH is the lane's pair
     static_assert(L % 2 == 0 && NP <= NR, "block length");
     uint32_t P[NR];
 #pragma unroll
@@ -159,20 +202,41 @@ __device__ __forceinline__ void flush_block(const uint32_t (&cum)[KH], uint32_t 
             P[0] += __shfl_xor_sync(0xffffffffu, P[0], o);
         }
     }
-    const uint32_t pi = NR == 32 ? (uint32_t)lane : (uint32_t)lane >> 1;    // this lane's pair
+    const uint32_t pi = (uint32_t)lane >> SH;               // this lane's pair
     const uint32_t t_lo = P[0] & 0xffffu, t_hi = P[0] >> 16;
     const uint32_t before = __reduce_add_sync(0xffffffffu, init_pop);       // total before the block
-    const uint32_t up_hi = __shfl_up_sync(0xffffffffu, t_hi, NR == 32 ? 1 : 2);
+    const uint32_t up_hi = __shfl_up_sync(0xffffffffu, t_hi, 1 << SH);
     const uint32_t prev = pi == 0 ? before : up_hi;
-    uint32_t cand = 0;
-    if (pi < (uint32_t)NP && (NR == 32 || (lane & 1) == 0)) {
+    if (pi < (uint32_t)NP && (lane & ((1 << SH) - 1)) == 0) {
         const uint32_t d_lo = t_lo - prev, d_hi = t_hi - t_lo;
-        if (d_lo) atomicAdd(&shist[K0 + 2 * pi + 1], d_lo);
-        if (d_hi) atomicAdd(&shist[K0 + 2 * pi + 2], d_hi);
-        cand = d_hi ? K0 + 2 * pi + 2 : d_lo ? K0 + 2 * pi + 1 : 0;
+        uint32_t* bins = first_bin + 2 * pi;
+        if (d_lo) atomicAdd(bins, d_lo);
+        if (d_hi) atomicAdd(bins + 1, d_hi);
     }
-    const uint32_t top = __reduce_max_sync(0xffffffffu, cand);
-    if (top) kmax = top;
+}
+
+// one step on one word of a later block: R1, R2 = windows of the merged words
+// of residue 1 and 2 (R[t] = word w - lo - t)
+template <int V, int I, int I0, int N1, int N2, int KH>
+__device__ __forceinline__ void later_step(const uint32_t (&R1)[N1], const uint32_t (&R2)[N2], uint32_t& C,
+                                           uint32_t (&cum)[KH], const uint32_t (&wt)[3])
+{
+    constexpr int rho = Step<V, I>::rho, t = Step<V, I>::c - Win<V, I0, kLater, rho>::lo;
+    constexpr uint32_t sh = Step<V, I>::sh;
+    uint32_t s;
+    if constexpr (rho == 1) s = sh == 0 ? R1[t] : __funnelshift_r(R1[t], R1[t > 0 ? t - 1 : 0], sh);
+    else s = sh == 0 ? R2[t] : __funnelshift_r(R2[t], R2[t > 0 ? t - 1 : 0], sh);
+    C |= s;
+    constexpr int j = I - I0;
+    cum[j / 3] = __popc(C) * wt[j % 3] + cum[j / 3];
+}
+
+template <int V, int I0, int N1, int N2, int KH, int... J>
+__device__ __forceinline__ void run_later(std::integer_sequence<int, J...>, const uint32_t (&R1)[N1],
+                                          const uint32_t (&R2)[N2], uint32_t& C, uint32_t (&cum)[KH],
+                                          const uint32_t (&wt)[3])
+{
+    (later_step<V, I0 + J, I0, N1, N2, KH>(R1, R2, C, cum, wt), ...);
 }
 
 // ---------------------------------------------------------------------------
@@ -182,67 +246,53 @@ __device__ __forceinline__ void flush_block(const uint32_t (&cum)[KH], uint32_t 
 // popc(C0) + popc(C1) + popc(C2) = popc(x) + 2 popc(y) with x the sum bits and
 // y the carry bits, two popcounts instead of three for two more logic ops
 // (the popcounts bound the step: measured 8.15 against 9.19 ms for the cover
-// of 2^34 even n near 5e11).
-// Window: R[t] = Q32[w + 2 + d_3/32 - t] for the lane's first word w.
-// ---------------------------------------------------------------------------
-__host__ __device__ constexpr int block0_regs3(int L0) { return (int)((step_e(L0 - 1) + 31) / 32) + 3; }
-
+// of 2^34 even n near 5e11, before the classes).
+// Window: R[t] = merged word w + 2 - t for the lane's first word w (block 0
+// starts at offset 0).
+//
 // The counts reach the 10-bit fields by integer multiply-adds with the field
 // weights 1, 2^10, 2^20 held as runtime values (not constants, which the
 // compiler would turn into shifts): the multiply-adds run on the FMA pipe and
 // leave the ALU pipe to the shifts and ORs, the popcounts run on the XU pipe.
-template <int K, int NR3, int KH>
-__device__ __forceinline__ void step3(const uint32_t (&R)[NR3], uint32_t& C0, uint32_t& C1, uint32_t& C2,
-                                      uint32_t (&cum)[KH], const uint32_t (&wt)[3])
+// ---------------------------------------------------------------------------
+template <int T, uint32_t SH, int N>
+__device__ __forceinline__ void or3(const uint32_t (&R)[N], uint32_t& C0, uint32_t& C1, uint32_t& C2)
 {
-    constexpr uint32_t e = step_e(K);
-    constexpr int c = (int)((e + 31) / 32);
-    constexpr uint32_t sh = 32 * c - e;
-    static_assert(c + 2 < NR3, "window too small");
-    uint32_t s0, s1, s2;
-    if constexpr (sh == 0) {
-        s0 = R[c + 2]; s1 = R[c + 1]; s2 = R[c];
+    static_assert(T + 2 < N, "window too small");
+    if constexpr (SH == 0) {
+        C0 |= R[T + 2];
+        C1 |= R[T + 1];
+        C2 |= R[T];
     } else {
-        s0 = __funnelshift_r(R[c + 2], R[c + 1], sh);
-        s1 = __funnelshift_r(R[c + 1], R[c], sh);
-        s2 = __funnelshift_r(R[c], R[c - 1], sh);
+        C0 |= __funnelshift_r(R[T + 2], R[T + 1], SH);
+        C1 |= __funnelshift_r(R[T + 1], R[T], SH);
+        C2 |= __funnelshift_r(R[T], R[T - 1], SH);
     }
-    C0 |= s0;
-    C1 |= s1;
-    C2 |= s2;
-    const uint32_t w = wt[K % 3];
+}
+
+template <int V, int I, int N1, int N2, int KH>
+__device__ __forceinline__ void step3(const uint32_t (&R1)[N1], const uint32_t (&R2)[N2], uint32_t& C0, uint32_t& C1,
+                                      uint32_t& C2, uint32_t (&cum)[KH], const uint32_t (&wt)[3])
+{
+    constexpr int t = Step<V, I>::c;
+    constexpr uint32_t sh = Step<V, I>::sh;
+    if constexpr (Step<V, I>::rho == 1) or3<t, sh>(R1, C0, C1, C2);
+    else or3<t, sh>(R2, C0, C1, C2);
+    const uint32_t w = wt[I % 3];
     const uint32_t x = C0 ^ C1 ^ C2;                        // sum bits
     const uint32_t y = (C0 & C1) | (C2 & (C0 | C1));        // carry bits (majority)
     const uint32_t py = __popc(y);
-    cum[K / 3] = __popc(x) * w + cum[K / 3];
-    cum[K / 3] = py * w + cum[K / 3];                       // twice: weight 2
-    cum[K / 3] = py * w + cum[K / 3];
+    cum[I / 3] = __popc(x) * w + cum[I / 3];
+    cum[I / 3] = py * w + cum[I / 3];                       // twice: weight 2
+    cum[I / 3] = py * w + cum[I / 3];
 }
 
-template <int NR3, int KH, int... J>
-__device__ __forceinline__ void run_block0_3(std::integer_sequence<int, J...>, const uint32_t (&R)[NR3], uint32_t& C0,
-                                             uint32_t& C1, uint32_t& C2, uint32_t (&cum)[KH], const uint32_t (&wt)[3])
+template <int V, int N1, int N2, int KH, int... J>
+__device__ __forceinline__ void run_block0(std::integer_sequence<int, J...>, const uint32_t (&R1)[N1],
+                                           const uint32_t (&R2)[N2], uint32_t& C0, uint32_t& C1, uint32_t& C2,
+                                           uint32_t (&cum)[KH], const uint32_t (&wt)[3])
 {
-    (step3<J, NR3, KH>(R, C0, C1, C2, cum, wt), ...);
-}
-
-// ---------------------------------------------------------------------------
-// tracked steps: record the last step that set a bit and the bits it set
-// ---------------------------------------------------------------------------
-template <int K, int K0, int NR>
-__device__ __forceinline__ void track_step(const uint32_t (&R)[NR], uint32_t& C, uint32_t& last, uint32_t& lastbits)
-{
-    const uint32_t s = window_shift<K, K0, NR>(R);
-    const uint32_t nw = s & ~C;
-    C |= s;
-    if (nw) { last = K + 1; lastbits = nw; }
-}
-
-template <int K0, int NR, int... J>
-__device__ __forceinline__ void track_block_steps(std::integer_sequence<int, J...>, const uint32_t (&R)[NR],
-                                                  uint32_t& C, uint32_t& last, uint32_t& lastbits)
-{
-    (track_step<K0 + J, K0, NR>(R, C, last, lastbits), ...);
+    (step3<V, J, N1, N2, KH>(R1, R2, C0, C1, C2, cum, wt), ...);
 }
 
 // a word of the q window: read-only global load, or a shared-memory load when
@@ -254,102 +304,91 @@ __device__ __forceinline__ uint32_t ldq(const uint32_t* p)
     else return __ldg(p);
 }
 
-// block (K0, L) on one word, tracked; C is updated.  The key of the word's
-// largest p_min within the block with its smallest n, 0 if the block set no bit
-template <int K0, int L, bool SQ>
-__device__ __forceinline__ unsigned long long track_word(const uint32_t* Qc, uint32_t D0w, uint32_t wrel, uint32_t& C,
-                                                         uint32_t j_cta)
+// what the functions below need of the chunk
+struct Chunk {
+    const uint32_t* Qc;         // window word of the chunk's first coverage word
+    const uint32_t* Y1;         // merged words of the q = 1 and = 2 (mod 3) in shared memory:
+    const uint32_t* Y2;         // Y[k] holds the partners of p = 3 for the merged n word k
+    uint32_t O;                 // words per stream
+    uint32_t o3;                // O mod 3 (1 or 2)
+    uint32_t na3;               // the chunk's first n, mod 3
+    uint32_t n_end;             // n of the chunk
+    uint32_t preset;            // bits of word 0: n = 4 and n = 6
+    uint64_t w_begin;           // the chunk's first word in the slab
+    uint32_t j_cta, seg;
+    uint32_t* lc;               // this warp's list: coverage, merged word index
+    uint16_t* lw;
+    uint32_t* shist;            // the CTA's bins [3][kMaxUseful]
+};
+
+// the n of the chunk's plain word W that are there to cover
+__device__ __forceinline__ uint32_t valid_bits(const Chunk& c, uint32_t W)
 {
-    constexpr int NR = block_regs(K0, L);
-    constexpr int C0 = block_c0(K0);
-    uint32_t R[NR];
-#pragma unroll
-    for (int t = 0; t < NR; ++t) R[t] = ldq<SQ>(Qc + wrel + D0w - C0 - t);
-    uint32_t last = 0, lastbits = 0;
-    track_block_steps<K0, NR>(std::make_integer_sequence<int, L>{}, R, C, last, lastbits);
-    if (!last) return 0;
-    const uint32_t j = j_cta + 32 * wrel + (__ffs(lastbits) - 1);
-    return ((unsigned long long)(last + 1) << 32) | (0xffffffffull - j);
+    const uint32_t j0 = 32 * W;
+    uint32_t v = j0 >= c.n_end ? 0u : c.n_end - j0 >= 32 ? 0xffffffffu : (1u << (c.n_end - j0)) - 1u;
+    if (W == 0) v &= ~c.preset;
+    return v;
 }
 
-// Later block K0 (kLater primes) over a warp's list [iw, ic) of n_in words, in
-// batches of 32 words (one per lane); the words still open go to [ow, oc),
-// which is either above the input or the input itself (then writes never pass
-// reads: each batch is read before its outputs land).
-template <int K0, bool SQ>
-__device__ __forceinline__ uint32_t later_block_warp(const uint32_t* Qc, uint32_t D0w, const uint16_t* iw,
-                                                     const uint32_t* ic, uint32_t n_in, uint16_t* ow, uint32_t* oc,
-                                                     uint32_t* shist, uint32_t& nsteps, uint32_t& kmax,
-                                                     const uint32_t (&wt)[3])
+// phase of the n = v (mod 3) in the chunk's plain word W: n = n_a + 2 (32 W + b)
+// = n_a + W + 2 b (mod 3), so b = 2 v + n_a + W
+__device__ __forceinline__ uint32_t n_phase(const Chunk& c, uint32_t v, uint32_t W) { return mod3(2 * v + c.na3 + W); }
+
+// coverage of merged word k of class v before the first prime: all but its valid n
+__device__ __forceinline__ uint32_t init_c(const Chunk& c, uint32_t v, uint32_t k)
+{
+    if (k >= c.O) return 0xffffffffu;
+    const uint32_t f = n_phase(c, v, k);
+    return ~((valid_bits(c, k) & phase_mask(f)) | (valid_bits(c, k + c.O) & phase_mask(mod3(f + c.o3))) |
+             (valid_bits(c, k + 2 * c.O) & phase_mask(mod3(f + 2 * c.o3))));
+}
+
+// The code of a chunk is kept small: of all that is unrolled, only the steps are
+// there once per class and block, behind uniform branches; the lists, the
+// counts' flush and the probing are there once (with everything unrolled per
+// class, 110 KB of code, the warps waited for instructions 60 % of the time and
+// the cover was slower than without the classes).
+
+// steps of block 0 of class v on the lane's words at .. at + 2
+template <int L0, int KH, int V>
+__device__ __forceinline__ void block0_class(const uint32_t* Y1, const uint32_t* Y2, uint32_t& C0, uint32_t& C1,
+                                             uint32_t& C2, uint32_t (&cum)[KH], const uint32_t (&wt)[3])
+{
+    static_assert(Win<V, 0, L0, 1>::lo == 0 && Win<V, 0, L0, 2>::lo == 0, "block 0 starts at offset 0");
+    constexpr int N1 = Win<V, 0, L0, 1>::n + 2, N2 = Win<V, 0, L0, 2>::n + 2;
+    uint32_t R1[N1], R2[N2];
+#pragma unroll
+    for (int t = 0; t < N1; ++t) R1[t] = Y1[2 - t];
+#pragma unroll
+    for (int t = 0; t < N2; ++t) R2[t] = Y2[2 - t];
+    run_block0<V, N1, N2, KH>(std::make_integer_sequence<int, L0>{}, R1, R2, C0, C1, C2, cum, wt);
+}
+
+// steps of the later block I0 of class V on one word
+template <int V, int I0, int KH>
+__device__ __forceinline__ void later_class(const uint32_t* Y1, const uint32_t* Y2, uint32_t& C, uint32_t (&cum)[KH],
+                                            const uint32_t (&wt)[3])
 {
     constexpr int L = kLater;
-    constexpr int NR = block_regs(K0, L);
-    constexpr int KH = (L + 2) / 3;
-    constexpr int C0 = block_c0(K0);
-    const int lane = threadIdx.x & 31;
-    uint32_t cum[KH];
+    constexpr int n1 = Win<V, I0, L, 1>::n, n2 = Win<V, I0, L, 2>::n, lo1 = Win<V, I0, L, 1>::lo, lo2 = Win<V, I0, L, 2>::lo;
+    constexpr int N1 = n1 ? n1 : 1, N2 = n2 ? n2 : 1;
+    uint32_t R1[N1], R2[N2];
+    R1[0] = R2[0] = 0;
 #pragma unroll
-    for (int j = 0; j < KH; ++j) cum[j] = 0;
-    uint32_t init_pop = 0, n_out = 0;
-    for (uint32_t b = 0; b < n_in; b += 32) {
-        const uint32_t e = b + lane;
-        const bool active = e < n_in;
-        uint32_t C = 0xffffffffu, wrel = 0;
-        uint32_t R[NR];
-        if (active) {
-            wrel = iw[e];
-            C = ic[e];
+    for (int t = 0; t < n1; ++t) R1[t] = Y1[-lo1 - t];
 #pragma unroll
-            for (int t = 0; t < NR; ++t) R[t] = ldq<SQ>(Qc + wrel + D0w - C0 - t);
-        } else {
-#pragma unroll
-            for (int t = 0; t < NR; ++t) R[t] = 0;
-        }
-        __syncwarp();                                      // the batch is read before outputs land
-        init_pop += __popc(C);
-        nsteps += active ? L : 0;
-        run_block<K0, NR, KH>(std::make_integer_sequence<int, L>{}, R, C, cum, wt);
-        const bool open = C != 0xffffffffu;
-        const unsigned m = __ballot_sync(0xffffffffu, open);
-        if (open) {
-            const uint32_t slot = n_out + __popc(m & ((1u << lane) - 1u));
-            ow[slot] = (uint16_t)wrel;
-            oc[slot] = C;
-        }
-        n_out += __popc(m);
-    }
-    __syncwarp();
-    flush_block<K0, L, KH>(cum, init_pop, shist, lane, kmax);
-    return n_out;
+    for (int t = 0; t < n2; ++t) R2[t] = Y2[-lo2 - t];
+    run_later<V, I0, N1, N2, KH>(std::make_integer_sequence<int, L>{}, R1, R2, C, cum, wt);
 }
 
-// later block b (1 .. kMaxLater) of a schedule with block 0 of L0 primes
-template <int L0, bool SQ, int B = 1>
-__device__ __forceinline__ uint32_t later_block_at(int b, const uint32_t* Qc, uint32_t D0w, const uint16_t* iw,
-                                                   const uint32_t* ic, uint32_t n_in, uint16_t* ow, uint32_t* oc,
-                                                   uint32_t* shist, uint32_t& nsteps, uint32_t& kmax,
-                                                   const uint32_t (&wt)[3])
+// later block b (from 1) of a schedule with block 0 of L0 primes
+template <int V, int L0, int KH, int B = 1>
+__device__ __forceinline__ void later_at(int b, const uint32_t* Y1, const uint32_t* Y2, uint32_t& C,
+                                         uint32_t (&cum)[KH], const uint32_t (&wt)[3])
 {
-    if constexpr (B > kMaxLater) {
-        return n_in;
-    } else {
-        if (b == B)
-            return later_block_warp<L0 + kLater * (B - 1), SQ>(Qc, D0w, iw, ic, n_in, ow, oc, shist, nsteps, kmax,
-                                                                  wt);
-        return later_block_at<L0, SQ, B + 1>(b, Qc, D0w, iw, ic, n_in, ow, oc, shist, nsteps, kmax, wt);
-    }
-}
-
-// later block b, tracked, on one word (C updated)
-template <int L0, bool SQ, int B = 1>
-__device__ __forceinline__ unsigned long long track_word_at(int b, const uint32_t* Qc, uint32_t D0w, uint32_t wrel,
-                                                            uint32_t& C, uint32_t j_cta)
-{
-    if constexpr (B > kMaxLater) {
-        return 0;
-    } else {
-        if (b == B) return track_word<L0 + kLater * (B - 1), kLater, SQ>(Qc, D0w, wrel, C, j_cta);
-        return track_word_at<L0, SQ, B + 1>(b, Qc, D0w, wrel, C, j_cta);
+    if constexpr (L0 + kLater * B <= kMaxUseful) {
+        if (b == B) later_class<V, L0 + kLater * (B - 1), KH>(Y1, Y2, C, cum, wt);
+        else later_at<V, L0, KH, B + 1>(b, Y1, Y2, C, cum, wt);
     }
 }
 
@@ -362,37 +401,45 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long ke
     return ((unsigned long long)mhi << 32) | mlo;
 }
 
+// bit b of merged word k of class v as a chunk-relative n index: the stream st
+// the bit came from has st O = b - f (mod 3), f the class's phase in word k
+__device__ __forceinline__ uint32_t merged_n(const Chunk& c, uint32_t f, uint32_t k, uint32_t b)
+{
+    const uint32_t d = mod3(b + 3 - f), st = c.o3 == 1 ? d : mod3(2 * d);
+    return 32 * (k + st * c.O) + b;
+}
+
 // Probing over a warp's list: the warp takes the open n one at a time, lane t
 // probing the prime k + t; the lowest set bit of the ballot is p_min.
 template <bool SQ>
-__device__ __forceinline__ void probe_warp(const CoverArgs& a, const uint32_t* Qc, const uint16_t* lw,
-                                           const uint32_t* lc, uint32_t n_in, uint32_t k_first, uint64_t w_begin,
-                                           uint32_t j_cta, uint32_t seg, unsigned long long& best, uint32_t& nsteps)
+__device__ __forceinline__ void probe_warp(const CoverArgs& a, const Chunk& c, uint32_t v, uint32_t n_in,
+                                           uint32_t k_first, unsigned long long& best, uint32_t& nsteps)
 {
     const int lane = threadIdx.x & 31;
     for (uint32_t e = 0; e < n_in; ++e) {
-        const uint32_t wrel = lw[e];
-        uint32_t mm = ~lc[e];
+        const uint32_t wk = c.lw[e];
+        const uint32_t f = n_phase(c, v, wk);
+        uint32_t mm = ~c.lc[e];
         while (mm) {
             const uint32_t b = __ffs(mm) - 1;
             mm &= mm - 1;
-            const uint32_t rel = 32 * wrel + b;              // CTA-relative n index
+            const uint32_t rel = merged_n(c, f, wk, b);      // CTA-relative n index
             uint32_t k = k_first;
             for (;;) {
                 const uint32_t kt = k + (uint32_t)lane;
                 uint32_t bit = 0;
                 if (kt < a.K) {
                     const uint32_t i = rel + ((a.H - __ldg(a.primes + 1 + kt) - 1) >> 1);
-                    bit = (ldq<SQ>(Qc + (i >> 5)) >> (i & 31)) & 1u;
+                    bit = (ldq<SQ>(c.Qc + (i >> 5)) >> (i & 31)) & 1u;
                 }
                 const unsigned hb = __ballot_sync(0xffffffffu, bit);
                 if (lane == 0) nsteps += 32;
                 if (hb) {
                     const uint32_t kk = k + (__ffs(hb) - 1);
                     if (lane == 0) {
-                        atomicAdd(&a.hist[(uint64_t)seg * a.hist_stride + kk + 1], 1u);
+                        atomicAdd(&a.hist[(uint64_t)c.seg * a.hist_stride + kk + 1], 1u);
                         const unsigned long long key =
-                            ((unsigned long long)(kk + 2) << 32) | (0xffffffffull - (j_cta + rel));
+                            ((unsigned long long)(kk + 2) << 32) | (0xffffffffull - (c.j_cta + rel));
                         if (key > best) best = key;
                     }
                     break;
@@ -401,7 +448,7 @@ __device__ __forceinline__ void probe_warp(const CoverArgs& a, const uint32_t* Q
                 if (k >= a.K) {
                     // open after every prime of this pass
                     if (lane == 0) {
-                        const uint64_t jn = 32 * w_begin + rel;          // slab-relative n index
+                        const uint64_t jn = 32 * c.w_begin + rel;        // slab-relative n index
                         bool queued = false;
                         if (a.retry) {
                             const unsigned int slot = atomicAdd(a.retry_count, 1u);
@@ -411,7 +458,7 @@ __device__ __forceinline__ void probe_warp(const CoverArgs& a, const uint32_t* Q
                                 queued = true;
                             }
                         }
-                        if (!queued) atomicAdd(&a.unresolved[seg], 1ull);
+                        if (!queued) atomicAdd(&a.unresolved[c.seg], 1ull);
                     }
                     break;
                 }
@@ -420,155 +467,272 @@ __device__ __forceinline__ void probe_warp(const CoverArgs& a, const uint32_t* Q
     }
 }
 
-// Block 0 of L0 primes over every word (three words per lane), up to
-// kMaxLater blocks of 32 over the words still open (a.n_later of them), then
-// per-n probing.  One chunk of coverage words [w_begin, w_end) (32-bit words
-// of the window a.Q, 32 even n each), all in segment (row) seg, whose first n
-// has segment-relative index j_cta.  Called by every thread of the CTA; smem
-// holds the per-warp lists; shist / smax are the CTA's shared counters.
-template <int NT, int L0, bool SQ>
-__device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* Qc, uint32_t seg, uint64_t w_begin,
-                                            uint64_t w_end, uint32_t j_cta, uint32_t* smem, uint32_t* shist,
-                                            unsigned long long& smax)
+// The largest p_min, with its smallest n, that the block of kLater useful primes
+// from I0 on gives the n open in the list (which it covers entirely, so that the
+// list is still there as it was before).
+__device__ __forceinline__ unsigned long long track_block(const Chunk& c, uint32_t v, uint32_t n_in, uint32_t I0)
 {
-    constexpr int NW = NT / 32;
+    unsigned long long best = 0;
+    for (uint32_t e = threadIdx.x & 31; e < n_in; e += 32) {
+        const uint32_t k = c.lw[e], f = n_phase(c, v, k);
+        uint32_t C = c.lc[e], last = 0, bits = 0;
+        for (uint32_t i = 0; i < (uint32_t)kLater; ++i) {
+            const uint32_t p = kClassDev.p[v][I0 + i], d = (p - 3) >> 1, w = (d + 31) >> 5;
+            const uint32_t* y = ((v + 3 - p % 3) % 3 == 1 ? c.Y1 : c.Y2) + k - w;
+            const uint32_t nw = ((d & 31) ? __funnelshift_r(y[0], y[1], 32 - (d & 31)) : y[0]) & ~C;
+            C |= nw;
+            if (nw) {
+                last = i + 1;
+                bits = nw;
+            }
+        }
+        if (!last) continue;
+        // the smallest n of the bits: of each stream's lowest
+        uint32_t n = 0xffffffffu;
+        for (uint32_t m = bits; m; m &= m - 1) n = min(n, merged_n(c, f, k, __ffs(m) - 1));
+        const unsigned long long key =
+            ((unsigned long long)(kClassDev.k[v][I0 + last - 1] + 2) << 32) | (0xffffffffull - (c.j_cta + n));
+        if (key > best) best = key;
+    }
+    return warp_max_key(best);
+}
+
+// Class v of a chunk: block 0 over the warp's merged words, the later blocks
+// over its open ones, probing.  best: the largest key of what block 0 left open
+// (0: none of that was covered); returns the odd-prime index of the blocks' last prime (an upper bound of the
+// others' p_min).
+template <int NW, int L0, bool SQ>
+__device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk& c, uint32_t v,
+                                                unsigned long long& best, uint32_t& nsteps, const uint32_t (&wt)[3])
+{
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t cap = list_cap(a.cta_words, NW);
-    uint32_t* lc = smem + (uint32_t)warp * cap;
-    uint16_t* lw = reinterpret_cast<uint16_t*>(smem + NW * cap) + (uint32_t)warp * cap;
-    const int n_later = (int)a.n_later;
-    const uint32_t prefix = (uint32_t)(L0 + kLater * n_later);
-    const uint32_t wt[3] = {a.cum_wt[0], a.cum_wt[1], a.cum_wt[2]};   // 1, 2^10, 2^20
-
-    __syncthreads();                                        // shared counters free (previous chunk)
-    for (uint32_t k = threadIdx.x; k <= prefix; k += NT) shist[k] = 0;
-    if (threadIdx.x == 0) smax = 0;
-    __syncthreads();
-
-    const uint32_t D0w = ((a.H - 4) >> 1) >> 5;            // word offset of the p = 3 partner
-    const uint32_t nw_cta = (uint32_t)(w_end > w_begin ? w_end - w_begin : 0);
-    const uint64_t n_left = a.n_count - 32 * w_begin;       // n from the CTA's first n to the window end
-    const uint32_t n_rel_end = (uint32_t)(n_left < 32ull * nw_cta ? n_left : 32ull * nw_cta);
-    // a word's coverage before the first prime: the lanes past the slab end,
-    // and n = 4 (= 2 + 2)
-    auto init_c = [&](uint32_t w) -> uint32_t {
-        uint32_t C = 0;
-        const uint32_t j0 = 32 * w;
-        if (n_rel_end - j0 < 32) C = 0xffffffffu << (n_rel_end - j0);
-        if (a.has_n4 && w_begin + w == 0) C |= 1u;
-        return C;
-    };
-
-    uint32_t nsteps = 0, n_open = 0, kmax = 0;
-    // block 0 over every word of this warp, three consecutive words per lane
+    uint32_t n_open = 0;
+    uint32_t* const bins = c.shist + v * kMaxUseful;
     {
-        constexpr int NR3 = block0_regs3(L0);
         constexpr int KH = (L0 + 2) / 3;
         uint32_t cum[KH];
 #pragma unroll
         for (int k = 0; k < KH; ++k) cum[k] = 0;
         uint32_t init_pop = 0;
-        for (uint32_t wbase = 96 * warp; wbase < nw_cta; wbase += 96 * NW) {
+        for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW) {
             const uint32_t wl = wbase + 3 * (uint32_t)lane;           // the lane's first word
-            uint32_t Cw[3];
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const uint32_t w = wl + i;
-                uint32_t C = 0xffffffffu;
-                if (w < nw_cta) {
-                    C = init_c(w);
-                    if (a.has_n4 && w_begin + w == 0) atomicAdd(&shist[0], 1u);
-                    nsteps += L0;
-                }
-                Cw[i] = C;
-                init_pop += __popc(C);
+            uint32_t C0 = 0, C1 = 0, C2 = 0;
+            if (wl + 2 >= c.O || 32 * (wl + 3 + 2 * c.O) > c.n_end || (wl == 0 && c.preset)) {
+                C0 = init_c(c, v, wl);
+                C1 = init_c(c, v, wl + 1);
+                C2 = init_c(c, v, wl + 2);
+                init_pop += __popc(C0) + __popc(C1) + __popc(C2);
             }
-            uint32_t R[NR3];
-            if (wl < nw_cta) {
-                // the top word read, wl + 2, lies at most one word past the CTA's
-                // last word: inside the q window, which runs past the slab
-#pragma unroll
-                for (int t = 0; t < NR3; ++t) R[t] = ldq<SQ>(Qc + wl + 2 + D0w - t);
-            } else {
-#pragma unroll
-                for (int t = 0; t < NR3; ++t) R[t] = 0;
-            }
-            uint32_t C0 = Cw[0], C1 = Cw[1], C2 = Cw[2];
-            run_block0_3<NR3, KH>(std::make_integer_sequence<int, L0>{}, R, C0, C1, C2, cum, wt);
-            Cw[0] = C0; Cw[1] = C1; Cw[2] = C2;
+            const bool active = wl < c.O;
+            nsteps += active ? 3 * L0 : 0;
+            // (a lane past the stream reads the window of word 0: its C are full)
+            const uint32_t at = active ? wl : 0;
+            const uint32_t *Y1 = c.Y1 + at, *Y2 = c.Y2 + at;
+            if (v == 0) block0_class<L0, KH, 0>(Y1, Y2, C0, C1, C2, cum, wt);
+            else if (v == 1) block0_class<L0, KH, 1>(Y1, Y2, C0, C1, C2, cum, wt);
+            else block0_class<L0, KH, 2>(Y1, Y2, C0, C1, C2, cum, wt);
+            const uint32_t Cw[3] = {C0, C1, C2};
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const bool open = Cw[i] != 0xffffffffu;
                 const unsigned m = __ballot_sync(0xffffffffu, open);
                 if (open) {
                     const uint32_t slot = n_open + __popc(m & ((1u << lane) - 1u));
-                    lw[slot] = (uint16_t)(wl + i);
-                    lc[slot] = Cw[i];
+                    c.lw[slot] = (uint16_t)(wl + i);
+                    c.lc[slot] = Cw[i];
                 }
                 n_open += __popc(m);
             }
         }
-        flush_block<0, L0, KH>(cum, init_pop, shist, lane, kmax);
+        flush_block<L0, KH>(cum, init_pop, bins, lane);
     }
     __syncwarp();
-
-    // later blocks; tb = the last block that set a bit, with its input list
-    int tb = 0;
-    uint32_t t_off = 0, t_n = 0;
-    bool t_kept = false;
-    uint32_t in_off = 0, n_cur = n_open;
-    int b_run = 0;
-    for (int b = 1; b <= n_later && n_cur > 0; ++b) {
-        const bool stack = in_off + 2 * n_cur <= cap;
-        const uint32_t out_off = stack ? in_off + n_cur : in_off;
-        const uint32_t kprev = kmax;
-        const uint32_t n_next = later_block_at<L0, SQ>(b, Qc, D0w, lw + in_off, lc + in_off, n_cur,
-                                                          lw + out_off, lc + out_off, shist, nsteps, kmax, wt);
-        if (kmax != kprev) {
-            tb = b;
-            t_off = in_off;
-            t_n = n_cur;
-            t_kept = stack;
-        }
-        in_off = out_off;
-        n_cur = n_next;
-        b_run = b;
-    }
-    unsigned long long best = 0;
-    probe_warp<SQ>(a, Qc, lw + in_off, lc + in_off, n_cur, (uint32_t)(L0 + kLater * b_run), w_begin, j_cta, seg,
-                   best, nsteps);
-
-    // the warp's largest p_min with its smallest n
-    unsigned long long wbest = warp_max_key(best);
-    if (wbest == 0 && kmax > 0) {
-        best = 0;
-        if (tb > 0 && t_kept) {
-            // block tb once more over its input list
-            for (uint32_t e = lane; e < t_n; e += 32) {
-                uint32_t C = lc[t_off + e];
-                const unsigned long long key = track_word_at<L0, SQ>(tb, Qc, D0w, lw[t_off + e], C, j_cta);
-                if (key > best) best = key;
+    // later blocks over the list, in batches of 32 words (one per lane); the
+    // words still open move up in it (each batch is read before its outputs land)
+    int b = 1;
+    for (; b <= (int)a.n_later && n_open > kProbeWords; ++b) {
+        constexpr int KH = (kLater + 2) / 3;
+        uint32_t cum[KH];
+#pragma unroll
+        for (int j = 0; j < KH; ++j) cum[j] = 0;
+        uint32_t init_pop = 0, n_out = 0;
+        for (uint32_t e0 = 0; e0 < n_open; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            const bool active = e < n_open;
+            uint32_t C = 0xffffffffu, k = 0;                // (an inactive lane reads word 0's window)
+            if (active) {
+                k = c.lw[e];
+                C = c.lc[e];
             }
-        } else {
-            // the warp's words through blocks 0 .. tb
-            for (uint32_t wbase = 96 * warp; wbase < nw_cta; wbase += 96 * NW) {
-                for (uint32_t w = wbase + lane; w < wbase + 96 && w < nw_cta; w += 32) {
-                    uint32_t C = init_c(w);
-                    unsigned long long key = track_word<0, L0, SQ>(Qc, D0w, w, C, j_cta);
-                    for (int b = 1; b <= tb; ++b) {
-                        const unsigned long long k2 = track_word_at<L0, SQ>(b, Qc, D0w, w, C, j_cta);
-                        if (k2 > key) key = k2;
-                    }
+            __syncwarp();
+            init_pop += __popc(C);
+            nsteps += active ? kLater : 0;
+            const uint32_t *Y1 = c.Y1 + k, *Y2 = c.Y2 + k;
+            if (v == 0) later_at<0, L0, KH>(b, Y1, Y2, C, cum, wt);
+            else if (v == 1) later_at<1, L0, KH>(b, Y1, Y2, C, cum, wt);
+            else later_at<2, L0, KH>(b, Y1, Y2, C, cum, wt);
+            const bool open = C != 0xffffffffu;
+            const unsigned m = __ballot_sync(0xffffffffu, open);
+            if (open) {
+                const uint32_t slot = n_out + __popc(m & ((1u << lane) - 1u));
+                c.lw[slot] = (uint16_t)k;
+                c.lc[slot] = C;
+            }
+            n_out += __popc(m);
+        }
+        __syncwarp();
+        flush_block<kLater, KH>(cum, init_pop, bins + L0 + kLater * (b - 1), lane);
+        if (n_out == 0) best = track_block(c, v, n_open, L0 + kLater * (b - 1));
+        n_open = n_out;
+    }
+    const uint32_t last = kClassDev.k[v][L0 + kLater * (b - 1) - 1];
+    probe_warp<SQ>(a, c, v, n_open, last + 1, best, nsteps);
+    __syncwarp();                                           // the list is the next class's
+    return last;
+}
+
+// The largest p_min among the first k_end + 1 odd primes, with its smallest n, of
+// the warp's words of class v: the plain words once more, one per lane.
+template <int NW, bool SQ>
+__device__ __forceinline__ unsigned long long recount_max(const CoverArgs& a, const Chunk& c, uint32_t v, uint32_t k_end)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long best = 0;
+    for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW)
+        for (uint32_t i = 0; i < 9; ++i) {
+            const uint32_t k = wbase + 32 * (i % 3) + lane, W = k + (i / 3) * c.O;
+            uint32_t open = k < c.O ? valid_bits(c, W) & phase_mask(n_phase(c, v, W)) : 0u;
+            for (uint32_t kk = 0; kk <= k_end && __any_sync(0xffffffffu, open != 0); ++kk) {
+                if (!open) continue;
+                const uint32_t d = (a.H - __ldg(a.primes + 1 + kk) - 1) >> 1;
+                const uint32_t* q = c.Qc + W + (d >> 5);
+                const uint32_t nw = ((d & 31) ? __funnelshift_r(ldq<SQ>(q), ldq<SQ>(q + 1), d & 31) : ldq<SQ>(q)) & open;
+                open &= ~nw;
+                if (nw) {
+                    const uint32_t j = c.j_cta + 32 * W + (__ffs(nw) - 1);
+                    const unsigned long long key = ((unsigned long long)(kk + 2) << 32) | (0xffffffffull - j);
                     if (key > best) best = key;
                 }
             }
         }
-        wbest = warp_max_key(best);
+    return warp_max_key(best);
+}
+
+// dynamic shared memory of a CTA: the merged words of both residues, then the
+// warps' lists
+struct CoverSmem {
+    uint32_t stream;            // words per stream, at most
+    uint32_t halo;              // merged words below a chunk's first
+    __host__ __device__ uint32_t merged() const { return (stream + halo + 2 + 3) & ~3u; }
+    __host__ __device__ uint32_t cap(int NW) const { return (stream + 96 * NW - 1) / (96 * NW) * 96; }
+    __host__ __device__ uint32_t bytes(int NW) const { return 8 * merged() + (uint32_t)NW * cap(NW) * 6; }
+};
+__host__ __device__ __forceinline__ uint32_t stream_words(uint32_t words)
+{
+    const uint32_t o = (words + 2) / 3;
+    return o % 3 == 0 ? o + 1 : o;
+}
+
+// shared counters of a CTA
+struct CoverShared {
+    uint32_t hist[3 * kMaxUseful];
+    unsigned long long smax;
+};
+
+// One chunk of coverage words [w_begin, w_end) (32-bit words of the window a.Q,
+// 32 even n each) whose first n is n0, all in segment (row) seg, where it has
+// index j_cta.  Qc is the window's word w_begin, of which words below q_lim may
+// be read.  Called by every thread of the CTA.
+template <int NT, int L0, bool SQ>
+__device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* Qc, uint32_t q_lim, uint64_t n0,
+                                            uint32_t seg, uint64_t w_begin, uint64_t w_end, uint32_t j_cta,
+                                            uint32_t* smem, CoverShared& sh)
+{
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const CoverSmem lay{stream_words(a.cta_words), a.halo_words};
+    const uint32_t nw_cta = (uint32_t)(w_end > w_begin ? w_end - w_begin : 0);
+    const uint32_t wt[3] = {a.cum_wt[0], a.cum_wt[1], a.cum_wt[2]};   // 1, 2^10, 2^20
+    uint32_t* const y1 = smem;
+    uint32_t* const y2 = smem + lay.merged();
+    uint32_t* const lists = smem + 2 * lay.merged();
+
+    Chunk c;
+    c.Qc = Qc;
+    c.Y1 = y1 + a.halo_words;
+    c.Y2 = y2 + a.halo_words;
+    c.O = stream_words(nw_cta);
+    c.o3 = c.O % 3;
+    c.na3 = (uint32_t)(n0 % 3);
+    const uint64_t n_left = nw_cta ? a.n_count - 32 * w_begin : 0;     // n from the chunk's first to the window end
+    c.n_end = (uint32_t)(n_left < 32ull * nw_cta ? n_left : 32ull * nw_cta);
+    c.preset = n0 == 4 ? 3u : n0 == 6 ? 1u : 0u;
+    c.w_begin = w_begin;
+    c.j_cta = j_cta;
+    c.seg = seg;
+    c.lc = lists + (uint32_t)warp * lay.cap(NW);
+    c.lw = reinterpret_cast<uint16_t*>(lists + NW * lay.cap(NW)) + (uint32_t)warp * lay.cap(NW);
+    c.shist = sh.hist;
+
+    __syncthreads();                                        // shared memory free (previous chunk)
+    for (uint32_t k = threadIdx.x; k < 3 * kMaxUseful; k += NT) sh.hist[k] = 0;
+    if (threadIdx.x == 0) sh.smax = 0;
+    {
+        // merged words: the window words of the three streams, from halo words
+        // below the first coverage word's partner of p = 3 on; q = Bc + 2 (32 W + b)
+        // with Bc = n0 - H + 1, so the bits of residue r are b = 2 r + Bc + W (mod 3)
+        const uint32_t base = (((a.H - 4) >> 1) >> 5) - a.halo_words;
+        const uint32_t bc3 = (c.na3 + 3u - a.H % 3u + 1u) % 3u;
+        const uint32_t total = c.O + a.halo_words + 2;
+        for (uint32_t t = threadIdx.x; t < total; t += NT) {
+            const uint32_t wa = base + t, wb = wa + c.O, wc = wb + c.O;
+            const uint32_t A = wa < q_lim ? ldq<SQ>(Qc + wa) : 0u, B = wb < q_lim ? ldq<SQ>(Qc + wb) : 0u,
+                           D = wc < q_lim ? ldq<SQ>(Qc + wc) : 0u;
+            const uint32_t f = mod3(2 + bc3 + wa);
+            const uint32_t m0 = phase_mask(f), m1 = phase_mask(mod3(f + 1)), m2 = ~(m0 | m1);    // phases f, f + 1, f + 2
+            // residue 1 has phase f in A, f + O in B, f + 2 O in D; residue 2 two more
+            const uint32_t B1 = c.o3 == 1 ? B : D, D1 = c.o3 == 1 ? D : B;
+            y1[t] = (A & m0) | (B1 & m1) | (D1 & m2);
+            y2[t] = (A & m2) | (B1 & m0) | (D1 & m1);
+        }
     }
-    if (lane == 0 && wbest) atomicMax(&smax, wbest);
     __syncthreads();
-    if (threadIdx.x == 0 && smax == 0 && a.has_n4 && w_begin == 0)
-        smax = (1ull << 32) | 0xffffffffull;               // only n = 4 (p_min 2, prime index 0)
+
+    uint32_t nsteps = 0;
+    uint32_t recount = 0;                                   // per class (10 bits): 1 + last prime's index where no n was probed
+#pragma unroll 1
+    for (uint32_t v = 0; v < 3; ++v) {
+        unsigned long long best = 0;
+        const uint32_t last = cover_class<NW, L0, SQ>(a, c, v, best, nsteps, wt);
+        best = __shfl_sync(0xffffffffu, best, 0);           // (the probing's lane)
+        if (best == 0) recount |= (last + 1) << (10 * v);
+        else if (lane == 0) atomicMax(&sh.smax, best);
+    }
+    if (threadIdx.x == 0 && c.preset) {
+        // n = 4 = 2 + 2 and n = 6 = 3 + 3
+        uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
+        if (n0 == 4) {
+            atomicAdd(&hrow[0], 1u);
+            atomicMax(&sh.smax, (1ull << 32) | (0xffffffffull - j_cta));
+        }
+        const uint32_t j6 = n0 == 4 ? 1u : 0u;
+        if (j6 < c.n_end) {
+            atomicAdd(&hrow[1], 1u);
+            atomicMax(&sh.smax, (2ull << 32) | (0xffffffffull - (j_cta + j6)));
+        }
+    }
+    __syncthreads();
+    // classes of which no n was probed: the maximum lies in the blocks
+#pragma unroll 1
+    for (uint32_t v = 0; v < 3 && recount; ++v) {
+        const uint32_t last1 = (recount >> (10 * v)) & 1023u;
+        const uint32_t top = (uint32_t)(*(volatile unsigned long long*)&sh.smax >> 32);
+        if (__any_sync(0xffffffffu, last1 && last1 + 1 >= top)) {
+            const unsigned long long key = recount_max<NW, SQ>(a, c, v, last1 - 1);
+            if (lane == 0 && key) atomicMax(&sh.smax, key);
+        }
+    }
+    __syncthreads();
 
     if (a.iters) {
         // unrolled word steps plus probes
@@ -577,38 +741,62 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
         if (lane == 0 && t) atomicAdd(a.iters, t);
     }
     uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
-    for (uint32_t kk = threadIdx.x; kk <= prefix; kk += NT)
-        if (shist[kk]) atomicAdd(&hrow[kk], shist[kk]);
-    if (threadIdx.x == 0 && smax) atomicMax(&a.maxkey[seg], smax);
+    for (uint32_t x = threadIdx.x; x < 3 * kMaxUseful; x += NT)
+        if (sh.hist[x]) atomicAdd(&hrow[kClassDev.k[x / kMaxUseful][x % kMaxUseful] + 1], sh.hist[x]);
+    if (threadIdx.x == 0 && sh.smax) atomicMax(&a.maxkey[seg], sh.smax);
 }
 
-// KA = L0 + 32 x (later blocks): L0 = 48 when KA = 16 (mod 32), else 64
-static bool split_prefix(int KA, int& L0, int& n_later)
+bool cover_prefix_valid(int KA) { return KA >= 48 && KA <= kMaxPrefix && KA % 16 == 0; }
+
+// block-cover fields of the arguments, and the length of block 0 (0: not to be
+// run).  The prefix KA counts primes; a class of n not divisible by 3 uses every
+// other one, so the blocks hold KA / 2 + 8 useful primes.  Block 0 takes 24 where
+// the pass has no more than the 48 primes that hold them, 48 near 1e17 and above
+// (KA = 240), 32 otherwise (2^33 n near 5e11: 2.69 ms with 28, 2.64 with 32, 2.67
+// with 36, 2.72 with 40; 2^31 near 1e15: 0.89, 0.87, 0.86, 0.85).
+static int cover_schedule(CoverArgs& a, int KA, int NW)
 {
-    if (KA < 48 || KA > kMaxPrefix || KA % 16 != 0) return false;
-    L0 = KA % 32 == 16 ? 48 : 64;
-    n_later = (KA - L0) / kLater;
-    return n_later <= kMaxLater;
+    if (!cover_prefix_valid(KA) || (uint32_t)KA > a.K || a.cta_words == 0) return 0;
+    if (stream_words(a.cta_words) > kMaxRounds * 96u * (uint32_t)NW) return 0;
+    auto fits = [&](int n) {                                // the first n useful primes of each class are in the pass
+        for (int v = 0; v < 3; ++v)
+            if (kClass.k[v][n - 1] >= a.K) return false;
+        return true;
+    };
+    const int L0 = KA >= 240 && fits(48) ? 48 : fits(32) ? 32 : fits(24) ? 24 : 0;
+    if (!L0) return 0;
+    int later = (KA / 2 + 8 - L0 + kLater - 1) / kLater;
+    while (later > 0 && (L0 + kLater * later > kMaxUseful || !fits(L0 + kLater * later))) --later;
+    a.n_later = (uint32_t)(later > 0 ? later : 0);
+    a.halo_words = 0;
+    for (int v = 0; v < 3; ++v)
+        a.halo_words = std::max<uint32_t>(a.halo_words, (uint32_t)use_c(v, L0 + kLater * (int)a.n_later - 1));
+    if (((a.H - 4) >> 6) < a.halo_words) return 0;
+    a.cum_wt[0] = 1; a.cum_wt[1] = 1u << kCumBits; a.cum_wt[2] = 1u << (2 * kCumBits);
+    return L0;
 }
 
 template <int NT, int L0>
-__global__ void __launch_bounds__(NT, 4) k_cover_fast(const CoverArgs a)
+__global__ void __launch_bounds__(NT, kCoverCtas) k_cover_fast(const CoverArgs a)
 {
-    extern __shared__ uint32_t smem[];                      // per warp: list C (32-bit), then words (16-bit)
-    __shared__ uint32_t shist[kMaxPrefix + 1];              // bins of the unrolled blocks' primes
-    __shared__ unsigned long long smax;
+    extern __shared__ uint32_t smem[];
+    __shared__ CoverShared sh;
     // this CTA's words, all in one segment
     const uint64_t wps = 2ull * a.words_per_seg;
     const uint32_t seg = blockIdx.x / a.chunks_per_seg;
     const uint32_t chunk = blockIdx.x % a.chunks_per_seg;
     const uint64_t seg_w0 = (uint64_t)seg * wps;
-    const uint64_t w_begin = seg_w0 + (uint64_t)chunk * (2ull * a.cta_words);
-    uint64_t w_end = w_begin + 2ull * a.cta_words;
+    const uint64_t w_begin = seg_w0 + (uint64_t)chunk * a.cta_words;
+    uint64_t w_end = w_begin + a.cta_words;
     const uint64_t n_words32 = (a.n_count + 31) / 32;
     if (w_end > seg_w0 + wps) w_end = seg_w0 + wps;
     if (w_end > n_words32) w_end = n_words32;
-    cover_chunk<NT, L0, false>(a, reinterpret_cast<const uint32_t*>(a.Q) + w_begin, seg, w_begin, w_end,
-                                  (uint32_t)(32 * (w_begin - seg_w0)), smem, shist, smax);
+    if (w_begin >= w_end) return;
+    const uint64_t q_words = 2 * (a.n_words + a.H / 128 + 2);
+    const uint64_t lim = q_words - w_begin;
+    cover_chunk<NT, L0, false>(a, reinterpret_cast<const uint32_t*>(a.Q) + w_begin,
+                               lim < 0xffffffffull ? (uint32_t)lim : 0xffffffffu, a.A0 + 64 * w_begin, seg, w_begin, w_end,
+                               (uint32_t)(32 * (w_begin - seg_w0)), smem, sh);
 }
 
 // Sieve and cover fused per CTA: the CTA sieves the q bits its chunk of
@@ -620,44 +808,31 @@ __global__ void __launch_bounds__(NT, 4) k_cover_fast(const CoverArgs a)
 template <int NT, int L0>
 __global__ void __launch_bounds__(NT, 2) k_seg_cover(const CoverArgs a, const SieveArgs sv, uint32_t off_w)
 {
-    extern __shared__ uint32_t smem[];                      // [lists | stamp tables | tile]
-    __shared__ uint32_t shist[kMaxPrefix + 1];
-    __shared__ unsigned long long smax;
+    extern __shared__ uint32_t smem[];                      // [cover | stamp tables | tile]
+    __shared__ CoverShared sh;
     constexpr int NW = NT / 32;
-    const uint32_t cap = list_cap(a.cta_words, NW);
-    uint32_t* lists = smem;
-    uint32_t* wt = smem + (NW * cap * 6) / 4;
+    const CoverSmem lay{stream_words(a.cta_words), a.halo_words};
+    uint32_t* wt = smem + ((lay.bytes(NW) / 4 + 3) & ~3u);
     uint32_t* tile = wt + ((kWheelWords + 3 + 3) & ~3u);    // 16-byte aligned
     const uint64_t wps = 2ull * a.words_per_seg;
     const uint32_t seg = blockIdx.x / a.chunks_per_seg;
     const uint32_t chunk = blockIdx.x % a.chunks_per_seg;
     const uint64_t seg_w0 = (uint64_t)seg * wps;
-    const uint64_t w_begin = seg_w0 + (uint64_t)chunk * (2ull * a.cta_words);
-    uint64_t w_end = w_begin + 2ull * a.cta_words;
+    const uint64_t w_begin = seg_w0 + (uint64_t)chunk * a.cta_words;
+    uint64_t w_end = w_begin + a.cta_words;
     const uint64_t n_words32 = (a.n_count + 31) / 32;
     if (w_end > seg_w0 + wps) w_end = seg_w0 + wps;
     if (w_end > n_words32) w_end = n_words32;
+    if (w_begin >= w_end) return;
     for (uint32_t i = threadIdx.x; i < kWheelWords; i += NT) wt[i] = sv.wheel[i];
     // tile word k is window word w_begin + off_w + k; the cover's Qc[k] is
     // window word w_begin + k and is only read at k >= off_w
-    sieve_tile<NT>(sv, 32ull * (w_begin + off_w), wt, tile);
-    cover_chunk<NT, L0, true>(a, tile - off_w, seg, w_begin, w_end, (uint32_t)(32 * (w_begin - seg_w0)), lists, shist,
-                              smax);
-}
-
-template <int L0>
-static cudaError_t launch_seg_l0(const CoverArgs& a, const SieveArgs& sv, uint32_t off_w, cudaStream_t s)
-{
-    constexpr int NT = 256;
-    const unsigned grid = a.nseg * a.chunks_per_seg;
-    if (grid == 0) return cudaSuccess;
-    const uint32_t cap = list_cap(a.cta_words, NT / 32);
-    const size_t smem = (size_t)(NT / 32) * cap * 6 + ((kWheelWords + 3 + 3) & ~3u) * 4 + kFusedTileBits / 8;
-    auto k = k_seg_cover<NT, L0>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k<<<grid, NT, smem, s>>>(a, sv, off_w);
-    return cudaGetLastError();
+    const uint64_t t0 = 32ull * (w_begin + off_w);
+    sieve_tile<NT>(sv, t0, wt, tile);
+    const uint64_t have = (sv.nbits - t0 + 31) / 32;
+    const uint32_t tile_words = have < kFusedTileBits / 32 ? (uint32_t)have : kFusedTileBits / 32;
+    cover_chunk<NT, L0, true>(a, tile - off_w, off_w + tile_words, a.A0 + 64 * w_begin, seg, w_begin, w_end,
+                              (uint32_t)(32 * (w_begin - seg_w0)), smem, sh);
 }
 
 uint32_t seg_cover_offset(uint32_t H, uint32_t P1)
@@ -666,31 +841,46 @@ uint32_t seg_cover_offset(uint32_t H, uint32_t P1)
     return bits >= 64 ? bits / 32 - 1 : 0;
 }
 
+template <int L0>
+static cudaError_t launch_seg_l0(const CoverArgs& a, const SieveArgs& sv, uint32_t off_w, cudaStream_t s)
+{
+    constexpr int NT = kFusedNT;
+    const unsigned grid = a.nseg * a.chunks_per_seg;
+    if (grid == 0) return cudaSuccess;
+    const CoverSmem lay{stream_words(a.cta_words), a.halo_words};
+    const size_t smem = (((size_t)lay.bytes(NT / 32) / 4 + 3) & ~size_t(3)) * 4 + ((kWheelWords + 3 + 3) & ~3u) * 4 +
+                        kFusedTileBits / 8;
+    auto k = k_seg_cover<NT, L0>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, NT, smem, s>>>(a, sv, off_w);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_seg_cover(const CoverArgs& a0, const SieveArgs& sv, int KA, uint32_t P1, cudaStream_t s)
 {
     // the tile must hold the chunk's words and the partner halo read past
     // them, from the offset of the pass's largest prime on
     const uint32_t off_w = seg_cover_offset(a0.H, P1);
-    const uint64_t need_words = 2ull * a0.cta_words + ((a0.H - 4) >> 6) + 3 - off_w;
+    const uint64_t need_words = a0.cta_words + ((a0.H - 4) >> 6) + 3 - off_w;
     if (need_words * 32 > kFusedTileBits || sv.tile_bits != kFusedTileBits || sv.out || sv.popcount)
         return cudaErrorInvalidValue;
-    if (2ull * a0.cta_words > 10ull * 768) return cudaErrorInvalidValue;
-    int L0 = 0, nl = 0;
-    if (!split_prefix(KA, L0, nl) || (uint32_t)KA > a0.K) return cudaErrorInvalidValue;
     CoverArgs a = a0;
-    a.n_later = (uint32_t)nl;
-    a.cum_wt[0] = 1; a.cum_wt[1] = 1u << kCumBits; a.cum_wt[2] = 1u << (2 * kCumBits);
-    return L0 == 48 ? launch_seg_l0<48>(a, sv, off_w, s) : launch_seg_l0<64>(a, sv, off_w, s);
+    switch (cover_schedule(a, KA, kFusedNT / 32)) {
+    case 24: return launch_seg_l0<24>(a, sv, off_w, s);
+    case 32: return launch_seg_l0<32>(a, sv, off_w, s);
+    case 48: return launch_seg_l0<48>(a, sv, off_w, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 // persistent: CTAs take (range, chunk) items from the queue until it is empty;
 // row r of the histograms, keys and counts is range r
 template <int NT, int L0>
-__global__ void __launch_bounds__(NT, 4) k_cover_items(const CoverItemsArgs a)
+__global__ void __launch_bounds__(NT, kCoverCtas) k_cover_items(const CoverItemsArgs a)
 {
     extern __shared__ uint32_t smem[];
-    __shared__ uint32_t shist[kMaxPrefix + 1];
-    __shared__ unsigned long long smax;
+    __shared__ CoverShared sh;
     __shared__ uint32_t s_item;
     const uint32_t n_items = *a.n_items;
     for (;;) {
@@ -702,76 +892,59 @@ __global__ void __launch_bounds__(NT, 4) k_cover_items(const CoverItemsArgs a)
         const uint32_t ri = a.item_range[item];
         const BatchRange r = a.ranges[ri];
         CoverArgs c = a.base;
-        c.Q = a.Q + r.q_off;
         c.n_count = r.n;
-        c.n_words = (r.n + 63) / 64;
-        c.has_n4 = (r.lo == 4);
-        const uint64_t w_begin = (uint64_t)a.item_chunk[item] * (2ull * c.cta_words);
-        uint64_t w_end = w_begin + 2ull * c.cta_words;
+        const uint64_t w_begin = (uint64_t)a.item_chunk[item] * c.cta_words;
+        uint64_t w_end = w_begin + c.cta_words;
         const uint64_t nw32 = (r.n + 31) / 32;
         if (w_end > nw32) w_end = nw32;
-        cover_chunk<NT, L0, false>(c, reinterpret_cast<const uint32_t*>(c.Q) + w_begin, ri, w_begin, w_end,
-                                   (uint32_t)(32 * w_begin), smem, shist, smax);
+        const uint64_t lim = r.nbits / 32 - w_begin;
+        cover_chunk<NT, L0, false>(c, reinterpret_cast<const uint32_t*>(a.Q + r.q_off) + w_begin,
+                                   lim < 0xffffffffull ? (uint32_t)lim : 0xffffffffu, r.lo + 64 * w_begin, ri, w_begin,
+                                   w_end, (uint32_t)(32 * w_begin), smem, sh);
     }
 }
 
 template <int L0>
 static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
 {
-    constexpr int NT = 256;
-    const uint32_t cap = list_cap(a.base.cta_words, NT / 32);
-    const size_t smem = (size_t)(NT / 32) * cap * 6;
+    constexpr int NT = kCoverNT;
+    const size_t smem = CoverSmem{stream_words(a.base.cta_words), a.base.halo_words}.bytes(NT / 32);
     auto k = k_cover_items<NT, L0>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0, per_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem)) != cudaSuccess) return e;
-    k<<<(unsigned)(sms * (per_sm > 0 ? per_sm : 1)), NT, smem, s>>>(a);
+    k<<<(unsigned)(device_sms() * (per_sm > 0 ? per_sm : 1)), NT, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_cover_items(const CoverItemsArgs& a0, int KA, cudaStream_t s)
 {
-    if (2ull * a0.base.cta_words > 10ull * 768) return cudaErrorInvalidValue;
-    int L0 = 0, nl = 0;
-    if (!split_prefix(KA, L0, nl) || (uint32_t)KA > a0.base.K) return cudaErrorInvalidValue;
     CoverItemsArgs a = a0;
-    a.base.n_later = (uint32_t)nl;
-    a.base.cum_wt[0] = 1; a.base.cum_wt[1] = 1u << kCumBits; a.base.cum_wt[2] = 1u << (2 * kCumBits);
-    return L0 == 48 ? launch_items_l0<48>(a, s) : launch_items_l0<64>(a, s);
-}
-
-bool cover_prefix_valid(int KA)
-{
-    int L0 = 0, nl = 0;
-    return split_prefix(KA, L0, nl);
+    switch (cover_schedule(a.base, KA, kCoverNT / 32)) {
+    case 24: return launch_items_l0<24>(a, s);
+    case 32: return launch_items_l0<32>(a, s);
+    case 48: return launch_items_l0<48>(a, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 int cover_fast_phase_primes(uint32_t K, uint64_t n_hi)
 {
-    // by magnitude (cover of 2^34 even n timed for KA = 112 .. 240 near 1e10,
-    // 1e11, 5e11, 1e13, 1e15 and 4e18): 48 + 3 x 32 primes below 1e14, 48 +
-    // 4 x 32 below 1e17, 48 + 6 x 32 above; the share of 32-n words still
-    // open after 48 primes is about 0.31 near 1e10, after 80 about 0.05, after
-    // 112 about 0.003
+    // by magnitude: 144 primes below 1e14, 176 below 1e17, 240 above
     int ka = n_hi < 100000000000000ull ? 144 : n_hi < 100000000000000000ull ? 176 : 240;
     while (ka >= 48 && (uint32_t)ka > K) ka -= 32;
-    if (ka < 48 && K >= 48) ka = 48;                        // the shortest schedule, block 0 alone
+    if (ka < 48 && K >= 48) ka = 48;                        // the shortest schedule
     return ka >= 48 ? ka : 0;
 }
 
 template <int L0>
 static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
 {
-    constexpr int NT = 256;
+    constexpr int NT = kCoverNT;
     const unsigned grid = a.nseg * a.chunks_per_seg;
     if (grid == 0) return cudaSuccess;
-    // one list per warp holding every word it takes in a sub-chunk: 32-bit
-    // coverage, 16-bit CTA-relative index
-    const uint32_t cap = list_cap(a.cta_words, NT / 32);
-    const size_t smem = (size_t)(NT / 32) * cap * 6;
+    const size_t smem = CoverSmem{stream_words(a.cta_words), a.halo_words}.bytes(NT / 32);
     auto k = k_cover_fast<NT, L0>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -781,16 +954,13 @@ static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
 
 cudaError_t launch_cover_fast(const CoverArgs& a0, int KA, cudaStream_t s)
 {
-    // 10-bit counters: in block 0 a lane adds at most 96 per step per round
-    // (three words), at most 10 rounds of 768 words; later blocks add at most
-    // 32 per listed word, at most 30 per lane
-    if (2ull * a0.cta_words > 10ull * 768) return cudaErrorInvalidValue;
-    int L0 = 0, nl = 0;
-    if (!split_prefix(KA, L0, nl) || (uint32_t)KA > a0.K) return cudaErrorInvalidValue;
     CoverArgs a = a0;
-    a.n_later = (uint32_t)nl;
-    a.cum_wt[0] = 1; a.cum_wt[1] = 1u << kCumBits; a.cum_wt[2] = 1u << (2 * kCumBits);
-    return L0 == 48 ? launch_l0<48>(a, s) : launch_l0<64>(a, s);
+    switch (cover_schedule(a, KA, kCoverNT / 32)) {
+    case 24: return launch_l0<24>(a, s);
+    case 32: return launch_l0<32>(a, s);
+    case 48: return launch_l0<48>(a, s);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace gb

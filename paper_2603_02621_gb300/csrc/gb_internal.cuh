@@ -238,8 +238,8 @@ struct CoverArgs {
     uint64_t n_count;           // even n in the slab
     uint64_t n_words;           // ceil(n_count / 64)
     uint32_t words_per_seg;     // S / 64
-    uint32_t cta_words;         // words per CTA (multiple of 32)
-    uint32_t chunks_per_seg;    // ceil(words_per_seg / cta_words)
+    uint32_t cta_words;         // words per CTA: 64-bit words for the generic cover, 32-bit words for the block cover
+    uint32_t chunks_per_seg;    // CTAs per segment
     uint32_t nseg;              // segments in the slab
     const uint32_t* primes;     // [2, 3, 5, ...]
     uint32_t K;                 // odd primes used: primes[1 .. K]
@@ -251,6 +251,7 @@ struct CoverArgs {
     RetryItem* retry;           // optional: words left with zero bits go here
     unsigned int* retry_count;
     uint32_t retry_cap;
+    uint64_t A0;                // the slab's first n
     int has_n4;                 // slab starts at n = 4 (p_min(4) = 2)
     unsigned long long* iters;  // optional: sum over words of the primes applied
                                 // until the word filled (work count)
@@ -258,17 +259,20 @@ struct CoverArgs {
     // segments whose key in maxkey_check is still 0 and writes it to maxkey
     int max_only;
     const unsigned long long* maxkey_check;
-    // block cover only (set by the launcher): blocks of 32 primes after block 0
-    uint32_t n_later;
+    // block cover only (set by the launcher)
+    uint32_t n_later;           // blocks after block 0
+    uint32_t halo_words;        // words below a word's partner of p = 3 that the blocks read
     uint32_t cum_wt[3];         // 1, 2^10, 2^20: weights of the packed 10-bit counters
 };
 cudaError_t launch_cover(const CoverArgs& a, int threads, cudaStream_t s);
 
-// Block cover (k_cover_fast): unrolled blocks, the first (48 or 64 primes)
-// over every 32-bit coverage word, each later one (32 primes) over the words
-// still open; then, in the same kernel, each n still open probes the primes
-// KA+1 .. K in order (KA = 48 or 64 + 32 x later blocks, at most 256; 48 when
-// KA = 16 mod 32).  Needs K >= KA, H = 4 (mod 64) and no p_min array.
+// Block cover (k_cover_fast): per residue class of n mod 3, unrolled blocks of
+// the primes useful to it, the first over every 32-bit coverage word, each later
+// one over the words still open; then, in the same kernel, each n still open
+// probes the remaining primes up to K in order.  KA (a multiple of 16 in [48,
+// 256]) is the number of primes before the probing.  Needs K >= KA, H = 4 (mod
+// 64), A0 and no p_min array.
+uint32_t cover_chunk_words(uint64_t words, bool fused);   // 32-bit words per CTA (CoverArgs::cta_words) for a call of `words`
 int cover_fast_phase_primes(uint32_t K, uint64_t n_hi);   // KA for K primes near n_hi (0: none)
 bool cover_prefix_valid(int KA);
 cudaError_t launch_cover_fast(const CoverArgs& a, int KA, cudaStream_t s);

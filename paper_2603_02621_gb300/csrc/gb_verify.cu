@@ -107,6 +107,7 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
         ca.retry = retry ? ctx->retry.as<gb::RetryItem>() : nullptr;
         ca.retry_count = retry ? ctx->retry_count.as<unsigned int>() : nullptr;
         ca.retry_cap = retry_cap;
+        ca.A0 = A0;
         ca.has_n4 = (A0 == 4);
         ca.iters = ctx->work_ptr(1);
         // two-phase kernel unless a p_min array is wanted (the generic kernel
@@ -114,10 +115,9 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
         int KA = (pm || ctx->generic_cover || cfg.cover_prefix == 1) ? 0 : gb::cover_fast_phase_primes(K1, A0 + 2 * n_count);
         if (KA && cfg.cover_prefix > 1 && cfg.cover_prefix <= K1) KA = (int)cfg.cover_prefix;
         if (KA) {
-            // block cover: 7680 32-bit words per CTA (ten rounds of 96 words per
-            // warp, the most its 10-bit counters allow)
-            ca.cta_words = std::min<uint32_t>(3840, (uint32_t)(S / 64));
-            ca.chunks_per_seg = (uint32_t)((S / 64 + ca.cta_words - 1) / ca.cta_words);
+            const uint32_t seg_words = (uint32_t)(S / 32);
+            ca.cta_words = std::min<uint32_t>(gb::cover_chunk_words((n_count + 31) / 32, ctx->fused), seg_words);
+            ca.chunks_per_seg = (seg_words + ca.cta_words - 1) / ca.cta_words;
         }
         // fused sieve + cover (GB_FUSED=1): block cover, no large primes, the
         // chunk plus its partner halo within one shared-memory tile
@@ -125,7 +125,7 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
         gb::SieveArgs fsv{};
         const uint32_t P1max = ctx->base->h_primes[K1];           // largest prime of the first pass
         if (ctx->fused && KA &&
-            (2ull * ca.cta_words + (H - 4) / 64 + 3 - gb::seg_cover_offset(H, P1max)) * 32 <= gb::kFusedTileBits) {
+            ((uint64_t)ca.cta_words + (H - 4) / 64 + 3 - gb::seg_cover_offset(H, P1max)) * 32 <= gb::kFusedTileBits) {
             uint64_t np = 0, nsmall = 0;
             if ((rc = tile_sieve_args(ctx, B, qw * 64, fsv, np, nsmall))) return rc;
             fused = np <= nsmall;
