@@ -46,6 +46,16 @@ int fill_defaults(gb_config& c)
     return GB_OK;
 }
 
+// A window of fewer tiles than two per SM is cut into shorter ones (a multiple
+// of 8192 bits), so that every SM takes part: the 5 million bits of [4, 1e7]
+// 27 -> 15.5 us; 2^16 n near 1e15 30 -> 16 us (and with the first pass's halo
+// alone, 82 thousand bits where there were 590).
+static uint32_t short_tile(uint32_t tile_bits, uint64_t nbits)
+{
+    const uint64_t want = (nbits / (2ull * gb::device_sms()) + 8191) / 8192 * 8192;
+    return (uint32_t)std::min<uint64_t>(tile_bits, std::max<uint64_t>(want, 8192));
+}
+
 // sieve the odd numbers B + 2i, i < nbits, into out (device words) or count only
 // tile-sieve arguments for the window (B, nbits): the primes below the split
 // (from 47 on; 3..43 are stamped); *np and *nsmall receive the count of
@@ -60,7 +70,7 @@ int tile_sieve_args(gb_ctx* ctx, int64_t B, uint64_t nbits, gb::SieveArgs& a, ui
     a = gb::SieveArgs{};
     a.B = B;
     a.nbits = nbits;
-    a.tile_bits = ctx->cfg.tile_bits;
+    a.tile_bits = short_tile(ctx->cfg.tile_bits, nbits);
     a.primes = ctx->base->primes.as<uint32_t>() + gb::kFirstStrikeIdx;
     a.recip = ctx->base->recip.as<uint64_t>() + gb::kFirstStrikeIdx;
     const uint64_t nstrike = nsmall > gb::kFirstStrikeIdx ? nsmall - gb::kFirstStrikeIdx : 0;
@@ -162,7 +172,18 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
         const int64_t last = B + 2 * (int64_t)(nbits - 1);
         if (ctx->mid_limit > ctx->split(isqrt_u64((uint64_t)last))) {
             nmid = std::min<uint64_t>(np, std::max<uint64_t>(nsmall, ctx->pi(ctx->mid_limit - 1)));
-            if (nmid > nsmall) {
+            // a slice takes its CTA some 70 us whatever the window's length; its
+            // primes' strikes by atomics in L2 (0.33 a bit, 2.1e11 a second) take
+            // less while the slices are fewer than a sixth of the SMs
+            const uint64_t mid_slices = (nbits + gb::kMidSliceBits - 1) / gb::kMidSliceBits;
+            if (nmid > nsmall && mid_slices <= gb::device_sms() / 6) {
+                gb::LargeArgs ma = la;
+                ma.n_primes = (uint32_t)(nmid - nsmall);
+                ma.bit_lo = 0;
+                ma.bit_hi = nbits;
+                ma.sub_bits = 1u << 18;
+                GB_LAUNCH(gb::launch_large(ma, ctx->stream));
+            } else if (nmid > nsmall) {
                 gb::LargeArgs ma = la;
                 ma.n_primes = (uint32_t)(nmid - nsmall);
                 // starts from a residue table of the window (16 bytes per
@@ -499,9 +520,8 @@ void gb_destroy(gb_ctx* ctx)
     else cudaDeviceSynchronize();
     // the base primes are shared with the contexts made by gb_init_shared:
     // they are freed with the last context holding them (delete below)
-    DevBuf* bufs[] = {&ctx->q, &ctx->hist,
-                      &ctx->maxkey, &ctx->maxkey2, &ctx->unres, &ctx->retry, &ctx->retry_count, &ctx->summary,
-                      &ctx->rows, &ctx->merged, &ctx->pmin, &ctx->counter, &ctx->totals, &ctx->records, &ctx->work,
+    DevBuf* bufs[] = {&ctx->q, &ctx->slab, &ctx->retry, &ctx->summary,
+                      &ctx->rows, &ctx->merged, &ctx->pmin, &ctx->counter, &ctx->records, &ctx->work,
                       &ctx->bq, &ctx->bhist, &ctx->bkeys, &ctx->bunres, &ctx->bdesc, &ctx->brecords, &ctx->brows,
                       &ctx->qn, &ctx->qout, &ctx->blists, &ctx->bcounts, &ctx->bflags,
                       &ctx->cstate, &ctx->cring, &ctx->ccnt,

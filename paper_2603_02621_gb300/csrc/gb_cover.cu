@@ -30,6 +30,8 @@
 // cannot represent q = 2, so it is set directly.  Words still not full after
 // the first pass go to a retry list; the retry pass continues them with the
 // primes P1 < p <= P2 (Sec. 2.3.3's exhaustive fallback, run on the GPU).
+#include <algorithm>
+
 #include "gb_internal.cuh"
 
 namespace gb {
@@ -153,6 +155,17 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
     if (threadIdx.x == 0 && smax) atomicMax(&a.maxkey[seg], smax);
 }
 
+// 64-bit words per CTA: 2048, whose CTA fills its tables once for 64 words per
+// lane; for a call that would not give every SM two CTAs fewer, down to 256 (32
+// per warp of 256 threads): a warp's words are a serial chain of some hundred
+// primes.  [4, 1e7] with its p_min array: 39 CTAs 284 us, 306 CTAs
+// 65 us.
+uint32_t cover_generic_words(uint64_t words, uint64_t seg_words)
+{
+    const uint64_t want = (words / (2ull * device_sms()) + 31) / 32 * 32;
+    return (uint32_t)std::min<uint64_t>(std::min<uint64_t>(2048, seg_words), std::max<uint64_t>(want, 256));
+}
+
 cudaError_t launch_cover(const CoverArgs& a, int threads, cudaStream_t s)
 {
     const unsigned grid = a.nseg * a.chunks_per_seg;
@@ -187,6 +200,7 @@ cudaError_t launch_cover(const CoverArgs& a, int threads, cudaStream_t s)
 __global__ void __launch_bounds__(128) k_retry(const RetryArgs a)
 {
     const unsigned int n = min(*a.count, a.cap);
+    if (a.overflow && blockIdx.x == 0 && threadIdx.x == 0 && *a.count > a.cap) atomicAdd(a.overflow, *a.count - a.cap);
     for (unsigned int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         const uint64_t w = a.items[t].w;
         uint64_t C = a.items[t].C;
@@ -234,8 +248,7 @@ cudaError_t launch_retry(const RetryArgs& a, cudaStream_t s)
 __global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a)
 {
     const uint32_t seg = blockIdx.x;
-    unsigned long long key = a.maxkey[seg];
-    if (a.maxkey2 && a.maxkey2[seg] > key) key = a.maxkey2[seg];
+    const unsigned long long key = a.maxkey[seg];
     const uint32_t pidx1 = (uint32_t)(key >> 32);
     const uint32_t hl = pidx1;                      // entries >= hl are all zero
     const uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
@@ -272,7 +285,7 @@ cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t s)
 __global__ void __launch_bounds__(1024) k_finalize(const FinalizeArgs a)
 {
     unsigned long long unres = 0, best = 0;        // best: p << 32 | (0xffffffff - seg)
-    for (uint32_t k = threadIdx.x; k < a.nseg; k += 1024) {
+    for (uint32_t k = threadIdx.x; k < a.nseg; k += blockDim.x) {
         const SegSummary g = a.summary[k];
         unres += g.unresolved;
         if (g.max_pmin) {
@@ -294,8 +307,8 @@ __global__ void __launch_bounds__(1024) k_finalize(const FinalizeArgs a)
     __shared__ unsigned long long s_unres, s_best;
     if (threadIdx.x == 0) { s_unres = 0; s_best = 0; }
     __syncthreads();
-    atomicAdd(&s_unres, unres);
-    atomicMax(&s_best, best);
+    if (unres) atomicAdd(&s_unres, unres);
+    if (best) atomicMax(&s_best, best);
     __syncthreads();
     if (threadIdx.x == 0) {
         RangeTotals t{};
@@ -307,13 +320,15 @@ __global__ void __launch_bounds__(1024) k_finalize(const FinalizeArgs a)
             t.max_pmin_n = a.lo + 2 * (uint64_t)k * a.S + 2 * g.max_j;
             t.hist_len = g.hist_len;
         }
+        if (a.retry_count) t.open = *a.retry_count;
         *a.totals = t;
     }
 }
 
 cudaError_t launch_finalize(const FinalizeArgs& a, cudaStream_t s)
 {
-    k_finalize<<<1, 1024, 0, s>>>(a);
+    const unsigned threads = a.nseg >= 1024 ? 1024u : (a.nseg + 31) & ~31u;
+    k_finalize<<<1, threads ? threads : 32u, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -153,6 +153,7 @@ struct SieveArgs {
 struct LargeArgs {
     int64_t  B;                 // odd number of bit 0 of the window
     uint64_t bit_lo, bit_hi;    // chunk of the window to strike
+    uint64_t sub_bits;          // bits per row of the grid (0: the whole chunk in one)
     const uint32_t* primes;     // the large primes
     const uint64_t* recip;      // their Barrett reciprocals
     uint32_t n_primes;
@@ -264,6 +265,7 @@ struct CoverArgs {
     uint32_t halo_words;        // words below a word's partner of p = 3 that the blocks read
     uint32_t cum_wt[3];         // 1, 2^10, 2^20: weights of the packed 10-bit counters
 };
+uint32_t cover_generic_words(uint64_t words, uint64_t seg_words);   // cta_words of a call of `words` 64-bit words
 cudaError_t launch_cover(const CoverArgs& a, int threads, cudaStream_t s);
 
 // Block cover (k_cover_fast): per residue class of n mod 3, unrolled blocks of
@@ -298,6 +300,7 @@ struct RetryArgs {
     const RetryItem* items;
     const unsigned int* count;
     uint32_t cap;
+    unsigned int* overflow;     // optional: items that the list could not hold are added
 };
 cudaError_t launch_retry(const RetryArgs& a, cudaStream_t s);
 
@@ -315,7 +318,6 @@ struct ReduceArgs {
     uint32_t hist_stride;
     const uint32_t* hist;
     const unsigned long long* maxkey;
-    const unsigned long long* maxkey2;  // optional second key per segment (max-only pass)
     const unsigned long long* unresolved;
     const uint32_t* primes;
     SegSummary* summary;        // [nseg]
@@ -333,6 +335,8 @@ struct RangeTotals {
     unsigned long long max_pmin_n;
     uint32_t max_pmin;
     uint32_t hist_len;
+    uint32_t open;              // items of the retry list (FinalizeArgs::retry_count)
+    uint32_t reserved;
 };
 
 struct SegRecord {              // identical layout to gb_segment_result
@@ -347,6 +351,7 @@ struct FinalizeArgs {
     SegRecord* records;         // optional
     uint32_t nrecords;          // records written (<= nseg)
     RangeTotals* totals;
+    const unsigned int* retry_count;    // optional: copied to totals->open
 };
 cudaError_t launch_finalize(const FinalizeArgs& a, cudaStream_t s);
 

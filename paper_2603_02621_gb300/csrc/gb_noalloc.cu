@@ -164,7 +164,7 @@ extern "C" int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, ui
     ca.n_count = n_total;
     ca.n_words = n_words;
     ca.words_per_seg = (uint32_t)(S / 64);
-    ca.cta_words = (uint32_t)std::min<uint64_t>(2048, S / 64);
+    ca.cta_words = gb::cover_generic_words(n_words, S / 64);
     ca.chunks_per_seg = (uint32_t)((S / 64 + ca.cta_words - 1) / ca.cta_words);
     ca.nseg = 1;
     ca.primes = v.primes;
@@ -213,7 +213,6 @@ extern "C" int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, ui
     rd.hist_stride = hist_stride;
     rd.hist = hist;
     rd.maxkey = maxkey;
-    rd.maxkey2 = nullptr;
     rd.unresolved = unres;
     rd.primes = v.primes;
     rd.summary = summary;

@@ -149,7 +149,9 @@ struct gb_ctx {
     uint64_t L = 0;                   // primes are known up to L
     std::shared_ptr<BasePrimes> base = std::make_shared<BasePrimes>();
     DevBuf q;                         // slab q window
-    DevBuf hist, maxkey, maxkey2, unres, retry, retry_count, summary, rows, merged, pmin, counter, totals, records;
+    DevBuf slab;                      // a slab's zeroed arrays: segment keys, unresolved counts, retry count, histogram rows
+    DevBuf retry, summary, rows, pmin, counter, records;
+    DevBuf merged;                    // a call's totals (RangeHead), then the merged histogram
     DevBuf work;                      // profiling work counters: [0] sieve strikes, [1] cover iterations
     // batched mode
     DevBuf bq, bhist, bkeys, bunres, bdesc, brecords, brows;

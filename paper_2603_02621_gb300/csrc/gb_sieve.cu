@@ -201,6 +201,13 @@ cudaError_t launch_sieve(const SieveArgs& a, int threads, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// slice primes below this take the mod-30 wheel (their strikes per slice,
+// 1.75 * 2^20 / p, outnumber the wheel's start cost)
+#ifndef GB_MID_WHEEL_BELOW
+#define GB_MID_WHEEL_BELOW (1u << 16)
+#endif
+constexpr uint32_t kMidWheelBelow = GB_MID_WHEEL_BELOW;
+
 // ---------------------------------------------------------------------------
 // primes larger than a tile: each hits a tile at most once, so the tile kernel
 // would spend a Barrett start per (tile, prime) for at most one strike.  Here
@@ -208,11 +215,17 @@ cudaError_t launch_sieve(const SieveArgs& a, int threads, cudaStream_t s)
 // start per chunk) and clears its multiples in global memory with atomic AND;
 // a chunk of 2^28 bits (32 MB) keeps the struck words resident in L2.
 // ---------------------------------------------------------------------------
+// In a window too short to give every SM a slice, the slices' primes are struck
+// here too: a row of the grid takes one part of the window (sub_bits), so that a
+// small prime's many strikes are shared by several threads; below kMidWheelBelow
+// they step through the mod-30 wheel as in the slices.
 __global__ void __launch_bounds__(256) k_large(const LargeArgs a)
 {
-    const int64_t b = a.B + 2 * (int64_t)a.bit_lo;          // number of the chunk's first bit
-    const int64_t last = a.B + 2 * (int64_t)(a.bit_hi - 1);
-    const uint64_t span = a.bit_hi - a.bit_lo;
+    const uint64_t bit_lo = a.bit_lo + (uint64_t)blockIdx.y * a.sub_bits;
+    const uint64_t bit_hi = a.bit_hi - bit_lo < a.sub_bits ? a.bit_hi : bit_lo + a.sub_bits;
+    const int64_t b = a.B + 2 * (int64_t)bit_lo;            // number of the part's first bit
+    const int64_t last = a.B + 2 * (int64_t)(bit_hi - 1);
+    const uint64_t span = bit_hi - bit_lo;
     unsigned long long nstrike = 0;
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < a.n_primes; k += gridDim.x * blockDim.x) {
         const uint32_t p = a.primes[k];
@@ -223,10 +236,21 @@ __global__ void __launch_bounds__(256) k_large(const LargeArgs a)
             const uint64_t isq = ((uint64_t)((int64_t)pp - b)) >> 1;
             if (isq > i) i = isq;
         }
-        for (; i < span; i += p) {
-            const uint64_t bit = a.bit_lo + i;
+        if (i >= span) continue;
+        uint32_t g = 0x11111111u;                           // half gaps: every odd multiple
+        if (p < kMidWheelBelow) {
+            // only m p with m coprime to 30 (see kHalfGaps30)
+            const uint32_t pm = p % 30u;
+            const uint32_t inv = pm * pm % 30u * pm % 30u;
+            const uint32_t j = (pmod_u32(b, 30) + 2u * (uint32_t)(i % 15u)) % 30u * inv % 30u >> 1;
+            i += (uint64_t)p * ((kNextHalf30 >> (2 * j)) & 3u);
+            g = __funnelshift_r(kHalfGaps30, kHalfGaps30, 4 * ((uint32_t)(kNextPos30 >> (3 * j)) & 7u));
+        }
+        for (; i < span; g = __funnelshift_r(g, g, 4)) {
+            const uint64_t bit = bit_lo + i;
             if (GB_DCHECK(bit < a.bit_hi, kDbgLargeStrike))
                 atomicAnd(a.out + (bit >> 5), __funnelshift_l(0xfffffffeu, 0xfffffffeu, (uint32_t)bit));
+            i += (uint64_t)p * (g & 15u);
             ++nstrike;
         }
     }
@@ -236,12 +260,17 @@ __global__ void __launch_bounds__(256) k_large(const LargeArgs a)
     }
 }
 
-cudaError_t launch_large(const LargeArgs& a, cudaStream_t s)
+cudaError_t launch_large(const LargeArgs& a0, cudaStream_t s)
 {
-    if (a.n_primes == 0 || a.bit_hi <= a.bit_lo) return cudaSuccess;
+    if (a0.n_primes == 0 || a0.bit_hi <= a0.bit_lo) return cudaSuccess;
+    LargeArgs a = a0;
+    const uint64_t bits = a.bit_hi - a.bit_lo;
+    if (a.sub_bits == 0 || a.sub_bits > bits) a.sub_bits = bits;
+    const uint64_t rows = (bits + a.sub_bits - 1) / a.sub_bits;
+    if (rows > 65535) return cudaErrorInvalidValue;
     const uint32_t cap = device_sms() * 64u;
     const uint32_t grid = (a.n_primes + 255) / 256 < cap ? (a.n_primes + 255) / 256 : cap;
-    k_large<<<grid, 256, 0, s>>>(a);
+    k_large<<<dim3(grid, (unsigned)rows), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -257,13 +286,6 @@ cudaError_t launch_large(const LargeArgs& a, cudaStream_t s)
 // 2^33 (s < 2^13, p < 2^20) reduced by one 32-bit multiply-high with
 // floor(2^33 / p), whose quotient is at most two short (two conditional
 // subtractions), in place of the 64 x 64-bit product of the Barrett step.
-// slice primes below this take the mod-30 wheel (their strikes per slice,
-// 1.75 * 2^20 / p, outnumber the wheel's start cost)
-#ifndef GB_MID_WHEEL_BELOW
-#define GB_MID_WHEEL_BELOW (1u << 16)
-#endif
-constexpr uint32_t kMidWheelBelow = GB_MID_WHEEL_BELOW;
-
 // nw words from src to dst by the whole CTA: 16-byte vectors, several in
 // flight per thread, when both are 16-byte aligned (the slice is one CTA per
 // SM: its load and store are not hidden behind another CTA's strikes)

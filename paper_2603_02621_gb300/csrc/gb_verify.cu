@@ -6,6 +6,17 @@
 // results to the host at the end.
 #include "gb_runtime.cuh"
 
+// the first bytes of ctx->merged: what a call reads back besides its outputs;
+// the merged histogram follows
+struct RangeHead {
+    gb::RangeTotals totals;
+    unsigned int overflow;          // retry items that no list could hold
+    unsigned int reserved[7];
+};
+static_assert(sizeof(RangeHead) == 64, "layout");
+// histogram entries read back with the head (p_min up to 17863; more are copied apart)
+constexpr uint32_t kHeadHist = 2048;
+
 extern "C" {
 
 int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_result* out)
@@ -44,44 +55,53 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
     const bool segs_dev = out->segs && is_device_ptr(out->segs);
     const bool pmin_dev = out->pmin && is_device_ptr(out->pmin);
     int rc;
-    if ((rc = ctx->summary.ensure(nseg * sizeof(gb::SegSummary))) ||
-        (rc = ctx->merged.ensure((size_t)hist_stride * 8)) ||
-        (rc = ctx->totals.ensure(sizeof(gb::RangeTotals))) ||
+    const size_t merged_bytes = sizeof(RangeHead) + (size_t)hist_stride * 8;
+    if ((rc = ctx->summary.ensure(nseg * sizeof(gb::SegSummary))) || (rc = ctx->merged.ensure(merged_bytes)) ||
+        (rc = ctx->hstage.ensure(sizeof(RangeHead) + kHeadHist * 8)) ||
         (want_rows && !rows_dev && (rc = ctx->rows.ensure(std::max<uint64_t>(1, nseg * row_stride) * 8))) ||
         (out->segs && !segs_dev && (rc = ctx->records.ensure(nseg * sizeof(gb::SegRecord)))))
         return rc;
-    GB_CUDA(cudaMemsetAsync(ctx->merged.p, 0, (size_t)hist_stride * 8, s));
+    RangeHead* const d_head = ctx->merged.as<RangeHead>();
+    unsigned long long* const d_merged = reinterpret_cast<unsigned long long*>(d_head + 1);
+    GB_CUDA(cudaMemsetAsync(ctx->merged.p, 0, merged_bytes, s));
     uint64_t* rows_base = want_rows ? (rows_dev ? out->seg_hist : ctx->rows.as<uint64_t>()) : nullptr;
 
-    // per-slab buffers
+    // per-slab buffers; what starts at zero is one array: segment keys,
+    // unresolved counts, the retry list's count, histogram rows
     const uint64_t slab_n = std::min<uint64_t>(spb * S, n_total);
     const uint64_t slab_words = (slab_n + 63) / 64;
     const uint64_t slab_segs = std::min<uint64_t>(spb, nseg);
     const uint64_t q_words = slab_words + H / 128 + 2;
     const uint32_t retry_cap = (uint32_t)std::min<uint64_t>(slab_words, 1u << 21);
-    if ((rc = ctx->q.ensure(q_words * 8)) ||
-        (rc = ctx->hist.ensure(slab_segs * hist_stride * 4)) ||
-        (rc = ctx->maxkey.ensure(slab_segs * 8)) || (rc = ctx->maxkey2.ensure(slab_segs * 8)) ||
-        (rc = ctx->unres.ensure(slab_segs * 8)) ||
+    if ((rc = ctx->q.ensure(q_words * 8)) || (rc = ctx->slab.ensure(slab_segs * (16 + (size_t)hist_stride * 4) + 16)) ||
         (retry && (rc = ctx->retry.ensure((size_t)retry_cap * sizeof(gb::RetryItem)))) ||
-        (rc = ctx->retry_count.ensure(16)) ||
         (out->pmin && !pmin_dev && (rc = ctx->pmin.ensure(slab_n * 4))))
         return rc;
 
-    unsigned int overflow_total = 0;
+    // A short range is first sieved and covered with the first pass's halo; the
+    // retry pass, whose halo may be many times the range, sieves its window only
+    // when the first pass left some n open.  From P1 = 2^13 on that is rare (the
+    // largest p_min up to 4e18 is 9781), and a range of 2^22 n or more hardly
+    // notices the halo.
+    const uint32_t H1 = 64 * ((P1 + 1 - 4 + 63) / 64) + 4;
+    const bool lazy = retry && !ctx->fused && nseg <= spb && P1 >= (1u << 13) && n_total < (1u << 22);
+    const uint32_t Hc = lazy ? H1 : H;                    // halo of the cover's window
+
+    gb::ReduceArgs rd{};
+    gb::RetryArgs ra{};
     for (uint64_t s0 = 0; s0 < nseg; s0 += spb) {
         const uint64_t ns = std::min<uint64_t>(spb, nseg - s0);
         const uint64_t A0 = lo + 2 * s0 * S;
         const uint64_t n_count = std::min<uint64_t>(ns * S, n_total - s0 * S);
         const uint64_t n_words = (n_count + 63) / 64;
-        const uint64_t qw = n_words + H / 128 + 2;
-        const int64_t B = (int64_t)A0 - (int64_t)H + 1;
+        const uint64_t qw = n_words + Hc / 128 + 2;
+        const int64_t B = (int64_t)A0 - (int64_t)Hc + 1;
 
-        GB_CUDA(cudaMemsetAsync(ctx->hist.p, 0, ns * hist_stride * 4, s));
-        GB_CUDA(cudaMemsetAsync(ctx->maxkey.p, 0, ns * 8, s));
-        GB_CUDA(cudaMemsetAsync(ctx->maxkey2.p, 0, ns * 8, s));
-        GB_CUDA(cudaMemsetAsync(ctx->unres.p, 0, ns * 8, s));
-        GB_CUDA(cudaMemsetAsync(ctx->retry_count.p, 0, 16, s));
+        unsigned long long* const maxkey = ctx->slab.as<unsigned long long>();
+        unsigned long long* const unres = maxkey + ns;
+        unsigned int* const retry_count = reinterpret_cast<unsigned int*>(unres + ns);
+        uint32_t* const hist = retry_count + 4;
+        GB_CUDA(cudaMemsetAsync(ctx->slab.p, 0, ns * (16 + (size_t)hist_stride * 4) + 16, s));
         uint32_t* pm = nullptr;
         if (out->pmin) {
             pm = pmin_dev ? out->pmin + (s0 * S) : ctx->pmin.as<uint32_t>();
@@ -90,22 +110,22 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
 
         gb::CoverArgs ca{};
         ca.Q = ctx->q.as<uint64_t>();
-        ca.H = H;
+        ca.H = Hc;
         ca.n_count = n_count;
         ca.n_words = n_words;
         ca.words_per_seg = (uint32_t)(S / 64);
-        ca.cta_words = std::min<uint32_t>(2048, (uint32_t)(S / 64));
+        ca.cta_words = gb::cover_generic_words(n_words, S / 64);
         ca.chunks_per_seg = (uint32_t)((S / 64 + ca.cta_words - 1) / ca.cta_words);
         ca.nseg = (uint32_t)ns;
         ca.primes = ctx->base->primes.as<uint32_t>();
         ca.K = K1;
         ca.hist_stride = hist_stride;
-        ca.hist = ctx->hist.as<uint32_t>();
-        ca.maxkey = ctx->maxkey.as<unsigned long long>();
-        ca.unresolved = ctx->unres.as<unsigned long long>();
+        ca.hist = hist;
+        ca.maxkey = maxkey;
+        ca.unresolved = unres;
         ca.pmin = pm;
         ca.retry = retry ? ctx->retry.as<gb::RetryItem>() : nullptr;
-        ca.retry_count = retry ? ctx->retry_count.as<unsigned int>() : nullptr;
+        ca.retry_count = retry ? retry_count : nullptr;
         ca.retry_cap = retry_cap;
         ca.A0 = A0;
         ca.has_n4 = (A0 == 4);
@@ -146,15 +166,14 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
             // the retry pass reads Q from global memory: sieve the slab there
             // only if some word was left open
             unsigned int cnt = 0;
-            GB_CUDA(ctx->copy(&cnt, ctx->retry_count.p, 4, cudaMemcpyDeviceToHost, s));
+            GB_CUDA(ctx->copy(&cnt, retry_count, 4, cudaMemcpyDeviceToHost, s));
             GB_CUDA(cudaStreamSynchronize(s));
             if (cnt) {
                 if ((rc = run_sieve(ctx, B, qw * 64, ctx->q.as<uint32_t>(), nullptr))) return rc;
                 q_in_hbm = true;
             }
         }
-        if (retry && q_in_hbm) {
-            gb::RetryArgs ra{};
+        if (retry) {
             ra.Q = ca.Q;
             ra.H = H;
             ra.words_per_seg = ca.words_per_seg;
@@ -169,14 +188,15 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
             ra.items = ca.retry;
             ra.count = ca.retry_count;
             ra.cap = retry_cap;
-            ctx->prof_begin(kProfRetry, n_count);
-            GB_LAUNCH(gb::launch_retry(ra, s));
-            ctx->prof_end();
+            ra.overflow = &d_head->overflow;
+            if (q_in_hbm && !lazy) {
+                ctx->prof_begin(kProfRetry, n_count);
+                GB_LAUNCH(gb::launch_retry(ra, s));
+                ctx->prof_end();
+            }
         }
 
-        gb::ReduceArgs rd{};
         rd.nseg = (uint32_t)ns;
-        rd.maxkey2 = nullptr;
         rd.hist_stride = hist_stride;
         rd.hist = ca.hist;
         rd.maxkey = ca.maxkey;
@@ -186,31 +206,13 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
         rd.rows = (want_rows && s0 < rows_n) ? rows_base + s0 * row_stride : nullptr;
         rd.row_stride = row_stride;
         rd.nrows = (uint32_t)(want_rows ? std::min<uint64_t>(ns, rows_n > s0 ? rows_n - s0 : 0) : 0);
-        rd.merged = ctx->merged.as<unsigned long long>();
+        rd.merged = d_merged;
         ctx->prof_begin(kProfReduce, ns);
         GB_LAUNCH(gb::launch_reduce(rd, s));
         ctx->prof_end();
 
-        if (retry) {
-            unsigned int cnt = 0;
-            GB_CUDA(ctx->copy(&cnt, ctx->retry_count.p, 4, cudaMemcpyDeviceToHost, s));
-            GB_CUDA(cudaStreamSynchronize(s));
-            if (cnt > retry_cap) overflow_total += cnt - retry_cap;
-        }
-        if (out->pmin && !pmin_dev)
+        if (out->pmin && !pmin_dev && !lazy)
             GB_CUDA(ctx->copy(out->pmin + s0 * S, pm, n_count * 4, cudaMemcpyDeviceToHost, s));
-    }
-    if (overflow_total) {
-        // the retry list could not hold every word left open: redo in one pass to Pf
-        gb_range_result again = *out;
-        const uint32_t saved_p2 = ctx->cfg.p2;
-        ctx->cfg.p2 = 0;
-        rc = gb_verify_range(ctx, lo, hi, Pf, &again);
-        ctx->cfg.p2 = saved_p2;
-        if (rc && rc != GB_ERANGE) return rc;
-        again.p_final = Pf;
-        *out = again;
-        return rc;
     }
 
     gb::FinalizeArgs fa{};
@@ -222,22 +224,65 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
     fa.records = out->segs ? (segs_dev ? reinterpret_cast<gb::SegRecord*>(out->segs) : ctx->records.as<gb::SegRecord>())
                            : nullptr;
     fa.nrecords = (uint32_t)(out->segs ? std::min<uint64_t>(out->seg_cap, nseg) : 0);
-    fa.totals = ctx->totals.as<gb::RangeTotals>();
-    ctx->prof_begin(kProfReduce, nseg);
-    GB_LAUNCH(gb::launch_finalize(fa, s));
-    ctx->prof_end();
-
-    gb::RangeTotals tot{};
-    GB_CUDA(ctx->copy(&tot, ctx->totals.p, sizeof tot, cudaMemcpyDeviceToHost, s));
+    fa.totals = &d_head->totals;
+    fa.retry_count = lazy ? ra.count : nullptr;
+    // the totals, with the first histogram entries, to pinned memory
     const uint32_t nh = out->hist ? std::min<uint32_t>(out->hist_cap, hist_stride) : 0;
-    if (nh) GB_CUDA(ctx->copy(out->hist, ctx->merged.p, (size_t)nh * 8, cudaMemcpyDeviceToHost, s));
+    const uint32_t nh_head = std::min<uint32_t>(nh, kHeadHist);
+    RangeHead* const head = static_cast<RangeHead*>(ctx->hstage.p);
+    auto finish = [&]() -> int {
+        ctx->prof_begin(kProfReduce, nseg);
+        GB_LAUNCH(gb::launch_finalize(fa, s));
+        ctx->prof_end();
+        GB_CUDA(ctx->copy(head, d_head, sizeof *head + (size_t)nh_head * 8, cudaMemcpyDeviceToHost, s));
+        GB_CUDA(cudaStreamSynchronize(s));
+        return GB_OK;
+    };
+    if ((rc = finish())) return rc;
+    if (lazy && head->totals.open) {
+        // n left open: the window with the retry pass's halo, the retry pass, and
+        // the reductions once more
+        const uint64_t qw = (n_total + 63) / 64 + H / 128 + 2;
+        if ((rc = run_sieve(ctx, (int64_t)lo - (int64_t)H + 1, qw * 64, ctx->q.as<uint32_t>(), nullptr))) return rc;
+        ra.H = H;
+        ctx->prof_begin(kProfRetry, n_total);
+        GB_LAUNCH(gb::launch_retry(ra, s));
+        ctx->prof_end();
+        GB_CUDA(cudaMemsetAsync(d_merged, 0, (size_t)hist_stride * 8, s));
+        ctx->prof_begin(kProfReduce, nseg);
+        GB_LAUNCH(gb::launch_reduce(rd, s));
+        ctx->prof_end();
+        if ((rc = finish())) return rc;
+    }
+    if (head->overflow) {
+        // the retry list could not hold every word left open: redo in one pass to Pf
+        gb_range_result again = *out;
+        const uint32_t saved_p2 = ctx->cfg.p2;
+        ctx->cfg.p2 = 0;
+        rc = gb_verify_range(ctx, lo, hi, Pf, &again);
+        ctx->cfg.p2 = saved_p2;
+        if (rc && rc != GB_ERANGE) return rc;
+        again.p_final = Pf;
+        *out = again;
+        return rc;
+    }
+    if (out->pmin && !pmin_dev && lazy)
+        GB_CUDA(ctx->copy(out->pmin, ctx->pmin.p, n_total * 4, cudaMemcpyDeviceToHost, s));
+
+    const gb::RangeTotals tot = head->totals;
+    // histogram entries from hist_len on are zero
+    const uint32_t nh_used = std::min<uint32_t>(nh, tot.hist_len);
+    if (nh_used) std::memcpy(out->hist, head + 1, (size_t)std::min(nh_used, nh_head) * 8);
+    if (nh_used > nh_head)
+        GB_CUDA(ctx->copy(out->hist + nh_head, d_merged + nh_head, (size_t)(nh_used - nh_head) * 8,
+                          cudaMemcpyDeviceToHost, s));
     const uint64_t nrec = out->segs ? std::min<uint64_t>(out->seg_cap, nseg) : 0;
     if (nrec && !segs_dev)
         GB_CUDA(ctx->copy(out->segs, ctx->records.p, nrec * sizeof(gb::SegRecord), cudaMemcpyDeviceToHost, s));
     if (rows_n && !rows_dev)
         GB_CUDA(ctx->copy(out->seg_hist, ctx->rows.p, rows_n * row_stride * 8, cudaMemcpyDeviceToHost, s));
+    if (out->hist) std::memset(out->hist + nh_used, 0, (size_t)(out->hist_cap - nh_used) * 8);
     GB_CUDA(cudaStreamSynchronize(s));
-    if (out->hist) for (uint32_t i = nh; i < out->hist_cap; ++i) out->hist[i] = 0;
 
     out->n_checked = n_total;
     out->n_segments = (uint32_t)nseg;
