@@ -525,7 +525,7 @@ void gb_destroy(gb_ctx* ctx)
                       &ctx->bq, &ctx->bhist, &ctx->bkeys, &ctx->bunres, &ctx->bdesc, &ctx->brecords, &ctx->brows,
                       &ctx->qn, &ctx->qout, &ctx->blists, &ctx->bcounts, &ctx->bflags,
                       &ctx->cstate, &ctx->cring, &ctx->ccnt,
-                      &ctx->part_p, &ctx->part_rev, &ctx->part_out};
+                      &ctx->part_p, &ctx->part_rev, &ctx->part_out, &ctx->part_y, &ctx->part_z};
     for (DevBuf* b : bufs) b->release();
     delete ctx;
 }

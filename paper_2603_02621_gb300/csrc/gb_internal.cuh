@@ -499,7 +499,25 @@ struct PartitionArgs {
     uint64_t runs;              // word runs per n-block
     uint64_t run_words;         // words per run
     uint32_t* counts;           // [count], zeroed; r(n) added
+    uint64_t w_first;           // first word of the sums (those before are counted by k_part_corr)
+    int with_3_5;               // add the pairs of 3 and 5
 };
+// Pairs i < 480 O of many n by residues mod 15 (gb_partitions.cu)
+struct PartCorrArgs {
+    const uint32_t* P;          // as above
+    uint64_t m_min, m_max;      // (n - 2) / 2 of the first and the last n
+    uint32_t O;                 // words per stream, prime to 15, 480 O <= m_min / 2 + 1
+    uint32_t ny, nz;            // merged words per residue: O up to a multiple of 96; ny + 15 blocks + 17 or more
+    uint32_t* y;                // [8][ny]
+    uint32_t* z;                // [8][nz]
+    uint32_t run_words;         // merged words per warp, a multiple of 96
+    uint32_t* counts;           // [m_max - m_min + 1], added to
+    // set by the launcher
+    uint32_t blocks, runs;      // blocks of 480 m (32 n of each m mod 15), runs
+    uint32_t w1, w2;            // 1 and 2, weights of the counters' multiply-adds
+};
+uint64_t part_stream_words(uint64_t i_end);     // O for sums to i_end (0: too short)
+cudaError_t launch_part_corr(const PartCorrArgs& a, cudaStream_t s);
 cudaError_t launch_reverse_bits(const uint32_t* P, uint32_t* rev, uint64_t words, cudaStream_t s);
 cudaError_t launch_partitions(const PartitionArgs& a, cudaStream_t s);
 

@@ -97,14 +97,50 @@ int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts)
     pa.P = ctx->part_p.as<uint32_t>();
     pa.rev = ctx->part_rev.as<uint32_t>();
     pa.words = words;
-    pa.lo = lo;
-    pa.count = count;
-    pa.n_blocks = (count + 31) / 32;
     pa.run_words = 4096;
-    pa.counts = d_out;
-    const uint64_t need = ((hi - 4) / 2) / 2 / 32 + 1;                  // words of the largest n
-    pa.runs = (need + pa.run_words - 1) / pa.run_words;
-    GB_LAUNCH(gb::launch_partitions(pa, s));
+    // Sums over many words for more than two warps of n go by residues mod 15, a
+    // sixty-fourth of the way to the next multiple of lo at a time (the i up to
+    // the first n's half are common to all, the rest is left to the plain
+    // kernel); a residue's n come in blocks of 32, so fewer than 96 n would
+    // mostly fill them with none (about 64 is where the two meet).
+    for (uint64_t a = lo; a < hi;) {
+        const uint64_t m_min = (a - 2) / 2;
+        uint64_t b = hi;
+        uint64_t O = 0;
+        if (a < (1u << 20)) b = std::min<uint64_t>(hi, 1u << 20);       // short sums: the plain kernel
+        if (a >= (1u << 20) && (hi - a) / 2 >= 96) {
+            b = std::min(hi, a + std::max<uint64_t>(960, a / 64 / 2 * 2));
+            if (hi - b < 192) b = hi;
+            O = gb::part_stream_words(m_min / 2 + 1);
+        }
+        if (O) {
+            gb::PartCorrArgs ca{};
+            ca.P = pa.P;
+            ca.m_min = m_min;
+            ca.m_max = (b - 4) / 2;
+            ca.O = (uint32_t)O;
+            ca.ny = (uint32_t)((O + 95) / 96 * 96);
+            const uint64_t blocks = (ca.m_max - m_min) / 480 + 1;
+            ca.nz = (uint32_t)(ca.ny + 15 * blocks + 17);
+            ca.run_words = 96 * 16;
+            if ((rc = ctx->part_y.ensure(32ull * ca.ny)) || (rc = ctx->part_z.ensure(32ull * ca.nz))) return rc;
+            ca.y = ctx->part_y.as<uint32_t>();
+            ca.z = ctx->part_z.as<uint32_t>();
+            ca.counts = d_out + (a - lo) / 2;
+            GB_LAUNCH(gb::launch_part_corr(ca, s));
+            ctx->kernels += 1;                                          // (two kernels)
+        }
+        pa.lo = a;
+        pa.count = (b - a) / 2;
+        pa.n_blocks = (pa.count + 31) / 32;
+        pa.counts = d_out + (a - lo) / 2;
+        pa.w_first = 15 * O;
+        pa.with_3_5 = O != 0;
+        const uint64_t need = ((b - 4) / 2) / 2 / 32 + 1 - pa.w_first;  // words of the largest n
+        pa.runs = std::max<uint64_t>(1, (need + pa.run_words - 1) / pa.run_words);
+        GB_LAUNCH(gb::launch_partitions(pa, s));
+        a = b;
+    }
     if (!out_dev) GB_CUDA(ctx->copy(counts, d_out, count * 4, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
     return GB_OK;

@@ -157,6 +157,7 @@ struct gb_ctx {
     DevBuf bq, bhist, bkeys, bunres, bdesc, brecords, brows;
     DevBuf qn, qout;                  // single-n queries: inputs, outputs + invalid-n counter
     DevBuf part_p, part_rev, part_out;  // partition counts: prime bits, reversed bits, counts
+    DevBuf part_y, part_z;            // and merged words by residue mod 15
     HostBuf hstage;
     bool batch_graph = true;          // batch kernels as one CUDA graph (GB_BATCH_GRAPH=0: plain launches)
     // bucket sieve of the primes >= 2^20 (GB_LARGE=bucket): per-tile hit
