@@ -151,12 +151,46 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
     uint64_t np = 0, nsmall = 0;
     int rc0 = tile_sieve_args(ctx, B, nbits, a, np, nsmall);
     if (rc0) return rc0;
+    // A long window with primes from 2^18 on, under the default tiling, goes
+    // through slabs: every prime below the slice limit in one pass.  From eight
+    // rounds of slabs on (2^30 odd numbers near 1e13, five rounds: 0.56 ms against
+    // 0.54 by tiles and slices; 2^31 near 1e15 2.26 against 2.29, large primes
+    // included).
+    const gb_config& c = ctx->cfg;
+    const int64_t last_num = B + 2 * (int64_t)(nbits - 1);
+    const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 36 && c.tile_bits == (1u << 18) &&
+                      c.bucket_split == 0 && c.cta_threads == 256 && ctx->mid_limit == (1u << 20) &&
+                      ctx->warp_split == 512 && nbits >= 8ull * gb::kSlabBits * gb::device_sms();
+    if (slab) nsmall = std::min<uint64_t>(np, ctx->pi((1u << 20) - 1));
     const bool large = np > nsmall && out;
     if (np > nsmall && !out) return fail(GB_EINVAL, "internal: large primes need an output buffer");
     a.out = out;
     a.popcount = large ? nullptr : popc;
     ctx->prof_begin(kProfSieve, nbits);
-    GB_LAUNCH(gb::launch_sieve(a, (int)ctx->cfg.cta_threads, ctx->stream));
+    if (slab) {
+        const uint64_t first = gb::kFirstStrikeIdx, n = nsmall > first ? nsmall - first : 0;
+        gb::SlabArgs sa{};
+        sa.B = B;
+        sa.nbits = nbits;
+        sa.primes = a.primes;
+        sa.recip = a.recip;
+        sa.n_primes = (uint32_t)n;
+        sa.n_warp = std::min(a.n_warp, sa.n_primes);
+        const uint64_t q = ctx->pi((1u << 13) - 1);
+        sa.n_quad = (uint32_t)std::min<uint64_t>(n, std::max<uint64_t>(sa.n_warp, q > first ? q - first : 0));
+        sa.wheel_below = 1u << 16;                        // (as in the slices)
+        const uint64_t wb = ctx->pi(sa.wheel_below - 1);
+        sa.n_plain = (uint32_t)std::min<uint64_t>(n, wb > first ? wb - first : 0);
+        const uint64_t pm = n ? ctx->base->h_primes[nsmall - 1] : 0;
+        sa.p_max2 = pm * pm;
+        sa.wheel = a.wheel;
+        sa.out = out;
+        sa.popcount = a.popcount;
+        sa.strikes = a.strikes;
+        GB_LAUNCH(gb::launch_slab(sa, ctx->stream));
+    } else {
+        GB_LAUNCH(gb::launch_sieve(a, (int)ctx->cfg.cta_threads, ctx->stream));
+    }
     ctx->prof_end();
     if (large) {
         ctx->prof_begin(kProfLarge, nbits);
@@ -168,9 +202,9 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
         la.out = out;
         la.strikes = ctx->work_ptr(2);
         // primes below mid_limit: per shared-memory slice of the window
-        uint64_t nmid = nsmall;
+        uint64_t nmid = nsmall;                             // (slabs: already past the slice limit)
         const int64_t last = B + 2 * (int64_t)(nbits - 1);
-        if (ctx->mid_limit > ctx->split(isqrt_u64((uint64_t)last))) {
+        if (!slab && ctx->mid_limit > ctx->split(isqrt_u64((uint64_t)last))) {
             nmid = std::min<uint64_t>(np, std::max<uint64_t>(nsmall, ctx->pi(ctx->mid_limit - 1)));
             // a slice takes its CTA some 70 us whatever the window's length; its
             // primes' strikes by atomics in L2 (0.33 a bit, 2.1e11 a second) take

@@ -176,6 +176,27 @@ constexpr uint32_t kMidSliceBits = 7u << 18;
 // slices per window for the residue starts (slice index x (2 kMidSliceBits mod p) < 2^33)
 constexpr uint32_t kMidResSlices = 1u << 13;
 cudaError_t launch_mid(const LargeArgs& a, uint64_t nbits, cudaStream_t s);
+// Segment sieve of a long window by every prime below 2^20 in one pass, one
+// shared-memory slab per CTA at a time (gb_slab.cu)
+constexpr uint32_t kSlabBits = 13u << 17;
+struct SlabArgs {
+    int64_t  B;                 // odd number of bit 0
+    uint64_t nbits;
+    const uint32_t* primes;     // sieving primes, ascending, starting at 47
+    const uint64_t* recip;      // their Barrett reciprocals
+    uint32_t n_warp;            // primes [0, n_warp): one warp strikes each
+    uint32_t n_quad;            // primes [n_quad, n_primes): four per thread at a time
+    uint32_t n_primes;
+    uint32_t wheel_below;       // one-thread primes below this step through the mod-30 wheel
+    uint32_t n_plain;           // primes [0, n_plain) are below wheel_below
+    uint64_t p_max2;            // square of the last prime
+    const uint32_t* wheel;      // the four stamp tables
+    uint32_t* out;              // NULL: count only
+    unsigned long long* popcount;   // optional total of 1 bits
+    unsigned long long* strikes;    // optional work count
+    uint32_t slab_bits;         // set by the launcher: the slabs' length, a multiple of 4096
+};
+cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s);
 // Primes from the slice limit to sqrt(B) over a window of several chunks of
 // 2^chunk_log2 bits (gb_large.cu): each prime started once per window and
 // carried from chunk to chunk -- per-prime next-multiple words for the primes
