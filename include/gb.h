@@ -62,7 +62,11 @@ typedef struct gb_config {
                                a segmented sieve of [A, B] needs primes to
                                sqrt(B)); 0 = 2^16; at most 2^32 */
     uint32_t tile_bits;     /* segment-sieve tile (odd numbers per CTA tile),
-                               multiple of 8192, <= 2^20; 0 = 2^18 */
+                               multiple of 8192, <= 2^20; 0 = 2^18.  Short
+                               windows are cut into shorter tiles; long ones
+                               go through slabs of up to 13 * 2^17 odd numbers
+                               while tile_bits, cta_threads and bucket_split
+                               are the defaults */
     uint32_t cta_threads;   /* threads per segment-sieve CTA: 128, 256 or
                                512; 0 = 256 */
     uint32_t bucket_split;  /* sieving primes >= this are struck by the
@@ -77,15 +81,15 @@ typedef struct gb_config {
     uint32_t p2;            /* retry-pass bound P2; 0 or <= p1 = no retry pass;
                                <= 2^24 */
     uint32_t cover_prefix;  /* primes of the cover's unrolled phase, a
-                               multiple of 16 in [48, 256]: a first block of
-                               48 (prefix = 16 mod 32) or 64 primes over every
-                               word, blocks of 32 over the words still open,
-                               then per-n probing; 0 = chosen by the magnitude
-                               of n; 1 = the generic cover (one 64-n word per
-                               lane, primes looped until the word is full),
-                               whose work counter is the algorithmic count.
-                               Outputs do not depend on it (the batched mode
-                               treats 1 as 0). */
+                               multiple of 16 in [48, 256]: per residue class of
+                               n mod 3 and over the primes useful to it, a first
+                               block over every word, then blocks of 16 over the
+                               words still open, then per-n probing; 0 = chosen
+                               by the magnitude of n; 1 = the generic cover (one
+                               64-n word per lane, primes looped until the word
+                               is full), whose work counter is the algorithmic
+                               count.  Outputs do not depend on it (the batched
+                               mode treats 1 as 0). */
     uint64_t slab_bits;     /* most q-bits sieved and kept resident at once
                                (a slab is a run of whole segments); 0 = 2^33 */
     void*    stream;        /* cudaStream_t for all work; NULL = the legacy
@@ -235,10 +239,10 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
  * for even n with 4 <= n < 2^63 (GB_EINVAL otherwise).  P is the context's
  * larger bound max(p1, p2).  Computed on the GPU: a window pre-sieve of the
  * partners n - p by the primes <= 2048, then a deterministic Miller-Rabin test
- * (bases 2..37) of each surviving partner, in ascending p.  Synchronous. */
+ * (bases 2..37) of the surviving partners, in ascending p.  Synchronous. */
 int gb_query(gb_ctx* ctx, uint64_t n, uint32_t* p_min);
 
-/* count queries at once (one CTA per n): n and p_min are host or device
+/* count queries at once (one warp per n): n and p_min are host or device
  * arrays of count entries; P as for gb_verify_range's bound (0: the context's
  * max(p1, p2)), at most the base primes.  Any invalid n gives GB_EINVAL (its
  * p_min is 0; the others are still computed).  Synchronous. */
@@ -298,7 +302,8 @@ void gb_server_destroy(gb_server* srv);
  * p + q = n (r(4) = 1, r(100) = 6).  Computed on the GPU from the odd-only
  * prime bitset of [1, hi) and its bit-reversed copy: for each n, popcount of
  * the AND of the bitset with the reversed one shifted to n, over p <= n/2
- * (about n/128 word steps per n).  lo even >= 4, hi even, hi <= 2^34 and
+ * (about n/128 word steps per n; 0.28 of them, by residues mod 30, from 96 n
+ * of 2^20 or more on).  lo even >= 4, hi even, hi <= 2^34 and
  * hi <= base_limit^2, at most 2^28 n per call; counts host or device.
  * Synchronous. */
 int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts);
@@ -336,7 +341,7 @@ int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P,
 
 /* Per-kernel device time, measured with CUDA events recorded on the
  * context's stream around every launch while profiling is enabled.  Kinds:
- * 0 segment sieve, tile part (units: q bits sieved), 1 cover (units: even n;
+ * 0 segment sieve, tile part or slabs (units: q bits sieved), 1 cover (units: even n;
  * batched mode: q bits), 2 retry pass (units: even n of the slabs it ran on),
  * 3 reductions and the max-only pass (units: segments), 4 segment sieve,
  * primes above the tile split (units: q bits).  gb_profile_enable resets the
@@ -351,7 +356,8 @@ int gb_profile_read(gb_ctx* ctx, double* ms, uint64_t* launches, uint64_t* units
 
 /* Work counted by the kernels while profiling is enabled: bits struck by the
  * segment sieve's tile part (every strike of a prime >= 47 below the tile
- * split, duplicates included; primes 3..43 are stamped from patterns); the
+ * split, or in slabs below 2^20, duplicates included; primes 3..43 are stamped
+ * from patterns); the
  * cover's steps: for the two-phase kernel, first-phase (32-bit word, prime)
  * steps plus second-phase (n, prime) probes; for the generic kernel, the sum
  * over 64-n words of the number of primes applied until the word filled (the

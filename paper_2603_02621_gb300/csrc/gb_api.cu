@@ -151,14 +151,14 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
     uint64_t np = 0, nsmall = 0;
     int rc0 = tile_sieve_args(ctx, B, nbits, a, np, nsmall);
     if (rc0) return rc0;
-    // A long window with primes from 2^18 on, under the default tiling, goes
+    // A long window with primes from 2^16 on, under the default tiling, goes
     // through slabs: every prime below the slice limit in one pass.  From eight
     // rounds of slabs on (2^30 odd numbers near 1e13, five rounds: 0.56 ms against
     // 0.54 by tiles and slices; 2^31 near 1e15 2.26 against 2.29, large primes
     // included).
     const gb_config& c = ctx->cfg;
     const int64_t last_num = B + 2 * (int64_t)(nbits - 1);
-    const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 36 && c.tile_bits == (1u << 18) &&
+    const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 32 && c.tile_bits == (1u << 18) &&
                       c.bucket_split == 0 && c.cta_threads == 256 && ctx->mid_limit == (1u << 20) &&
                       ctx->warp_split == 512 && nbits >= 8ull * gb::kSlabBits * gb::device_sms();
     if (slab) nsmall = std::min<uint64_t>(np, ctx->pi((1u << 20) - 1));
@@ -175,10 +175,16 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
         sa.primes = a.primes;
         sa.recip = a.recip;
         sa.n_primes = (uint32_t)n;
-        sa.n_warp = std::min(a.n_warp, sa.n_primes);
+        // primes below 512 a warp each; without primes from 2^18 on, and so with
+        // little other work in a slab, below 1024 (2^32 odd numbers from 4 on: 1.47
+        // ms with 512, 1.35 with 1024, 1.44 with 1536; near 5e11, 2^33: 3.53, 3.70,
+        // 3.95).  The work counters keep to 512, as the tiles.
+        const bool low = last_num < 1ll << 36;
+        const uint64_t nw = ctx->pi((low && !a.strikes ? 1024u : 512u) - 1);
+        sa.n_warp = (uint32_t)std::min<uint64_t>(n, nw > first ? nw - first : 0);
         const uint64_t q = ctx->pi((1u << 13) - 1);
         sa.n_quad = (uint32_t)std::min<uint64_t>(n, std::max<uint64_t>(sa.n_warp, q > first ? q - first : 0));
-        sa.wheel_below = 1u << 16;                        // (as in the slices)
+        sa.wheel_below = low ? 1u << 18 : 1u << 16;       // (as in the tiles; as in the slices)
         const uint64_t wb = ctx->pi(sa.wheel_below - 1);
         sa.n_plain = (uint32_t)std::min<uint64_t>(n, wb > first ? wb - first : 0);
         const uint64_t pm = n ? ctx->base->h_primes[nsmall - 1] : 0;

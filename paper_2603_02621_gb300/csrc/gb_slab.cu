@@ -7,16 +7,17 @@
 // Against tiles of 2^18 bits and slices of 1.75 * 2^20 read back from memory:
 // the window is written once and not read; a prime is started once per slab
 // instead of once per tile, or once more per slice; and a warp-struck prime
-// leaves each lane at least 104 strikes, so that all of them can start in
-// distinct banks (below).
+// leaves each lane enough strikes (104 and more below 512) that all of them can
+// start in distinct banks (below).
 //
 // Work inside a slab is taken from one queue by the warps, longest first, between
-// two barriers; a slab is stored and the next one stamped over it in one pass: primes below 512 one warp each,
-// then 32 primes to a warp (a thread each, up to 1700 strikes), then, from 2^13
-// on, 128 primes to a warp, four starts per thread overlapping.
+// two barriers: the smallest primes one warp each, then 32 primes to a warp (a
+// thread each, up to 1700 strikes), then, from 2^13 on, 128 primes to a warp,
+// four starts per thread overlapping.  A slab is stored and the next one stamped
+// over it in one pass.
 //
-// Bound: instruction issue and shared-memory wavefronts
-// together (68 and 73 % of their peaks at 5e11).  2^33 odd numbers near 5e11 on a
+// Bound: instruction issue and shared-memory wavefronts together (70 and 78 % of
+// their peaks at 5e11).  2^33 odd numbers near 5e11 on a
 // GB300: 3.77 ms by tiles and slices, 3.53 ms.  The strike loops are unrolled and
 // their ends masked rather than branched around: as plain loops, with a branch
 // per strike, the pass took 5.1 ms.

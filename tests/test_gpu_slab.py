@@ -29,7 +29,7 @@ def _sieve(gbm, A, nbits, **cfg):
     return n, q, w["sieve_strikes"] + w["large_strikes"]
 
 
-@pytest.mark.parametrize("A", [(1 << 37) + 1, 5 * 10**11 + 3, 10**12 - 10**9 + 1, 10**15 + 7])
+@pytest.mark.parametrize("A", [1, (1 << 33) + 5, (1 << 37) + 1, 5 * 10**11 + 3, 10**12 - 10**9 + 1, 10**15 + 7])
 @pytest.mark.parametrize("rounds,more", [(8, 0), (8, 1), (8, -64 + (1 << 18)), (9, 12345)])
 def test_slabs_equal_tiles_and_slices(gbm, A, rounds, more):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
