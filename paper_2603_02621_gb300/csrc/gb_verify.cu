@@ -54,6 +54,7 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
     const bool rows_dev = want_rows && is_device_ptr(out->seg_hist);
     const bool segs_dev = out->segs && is_device_ptr(out->segs);
     const bool pmin_dev = out->pmin && is_device_ptr(out->pmin);
+    const bool hist_dev = out->hist && is_device_ptr(out->hist);
     int rc;
     const size_t merged_bytes = sizeof(RangeHead) + (size_t)hist_stride * 8;
     if ((rc = ctx->summary.ensure(nseg * sizeof(gb::SegSummary))) || (rc = ctx->merged.ensure(merged_bytes)) ||
@@ -228,7 +229,7 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
     fa.retry_count = lazy ? ra.count : nullptr;
     // the totals, with the first histogram entries, to pinned memory
     const uint32_t nh = out->hist ? std::min<uint32_t>(out->hist_cap, hist_stride) : 0;
-    const uint32_t nh_head = std::min<uint32_t>(nh, kHeadHist);
+    const uint32_t nh_head = hist_dev ? 0 : std::min<uint32_t>(nh, kHeadHist);
     RangeHead* const head = static_cast<RangeHead*>(ctx->hstage.p);
     auto finish = [&]() -> int {
         ctx->prof_begin(kProfReduce, nseg);
@@ -270,18 +271,23 @@ int gb_verify_range(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P, gb_range_
         GB_CUDA(ctx->copy(out->pmin, ctx->pmin.p, n_total * 4, cudaMemcpyDeviceToHost, s));
 
     const gb::RangeTotals tot = head->totals;
-    // histogram entries from hist_len on are zero
+    // histogram entries from hist_len on are zero (a device buffer is filled in place)
     const uint32_t nh_used = std::min<uint32_t>(nh, tot.hist_len);
-    if (nh_used) std::memcpy(out->hist, head + 1, (size_t)std::min(nh_used, nh_head) * 8);
-    if (nh_used > nh_head)
-        GB_CUDA(ctx->copy(out->hist + nh_head, d_merged + nh_head, (size_t)(nh_used - nh_head) * 8,
-                          cudaMemcpyDeviceToHost, s));
+    if (hist_dev) {
+        GB_CUDA(cudaMemcpyAsync(out->hist, d_merged, (size_t)nh * 8, cudaMemcpyDeviceToDevice, s));
+        if (out->hist_cap > nh) GB_CUDA(cudaMemsetAsync(out->hist + nh, 0, (size_t)(out->hist_cap - nh) * 8, s));
+    } else if (nh_used) {
+        std::memcpy(out->hist, head + 1, (size_t)std::min(nh_used, nh_head) * 8);
+        if (nh_used > nh_head)
+            GB_CUDA(ctx->copy(out->hist + nh_head, d_merged + nh_head, (size_t)(nh_used - nh_head) * 8,
+                              cudaMemcpyDeviceToHost, s));
+    }
     const uint64_t nrec = out->segs ? std::min<uint64_t>(out->seg_cap, nseg) : 0;
     if (nrec && !segs_dev)
         GB_CUDA(ctx->copy(out->segs, ctx->records.p, nrec * sizeof(gb::SegRecord), cudaMemcpyDeviceToHost, s));
     if (rows_n && !rows_dev)
         GB_CUDA(ctx->copy(out->seg_hist, ctx->rows.p, rows_n * row_stride * 8, cudaMemcpyDeviceToHost, s));
-    if (out->hist) std::memset(out->hist + nh_used, 0, (size_t)(out->hist_cap - nh_used) * 8);
+    if (out->hist && !hist_dev) std::memset(out->hist + nh_used, 0, (size_t)(out->hist_cap - nh_used) * 8);
     GB_CUDA(cudaStreamSynchronize(s));
 
     out->n_checked = n_total;

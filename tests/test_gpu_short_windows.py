@@ -76,3 +76,21 @@ def test_slices_and_atomics_agree(gbm, monkeypatch, slices, tail):
     monkeypatch.setenv("GB_MID_LOG2", "0")
     pb, qb = sieve()
     assert pa == pb and torch.equal(qa, qb)
+
+
+@pytest.mark.parametrize("cap", [100, 3512, 100000])
+@pytest.mark.parametrize("n", [1000, 1 << 23])
+def test_histogram_into_device_memory(gbm, cap, n):
+    """The merged histogram into a device buffer of the caller: shorter than the
+    histogram's used part, longer, and longer than any prime index."""
+    import ctypes
+    lo = 10**12
+    with gbm.Context(device=0, base_limit=1 << 21, seg_len=1 << 20, p1=1 << 15, p2=1 << 20) as g:
+        want = g.verify_range(lo, lo + 2 * n, hist_cap=cap, allow_erange=True)
+        dev = torch.full((cap,), -1, dtype=torch.int64, device="cuda")
+        r = gbm.gb_range_result()
+        r.hist = ctypes.cast(dev.data_ptr(), ctypes.POINTER(ctypes.c_uint64))
+        r.hist_cap = cap
+        rc = gbm.load().gb_verify_range(g.handle, lo, lo + 2 * n, 0, ctypes.byref(r))
+    assert rc == want["rc"]
+    np.testing.assert_array_equal(dev.cpu().numpy().view(np.uint64), want["hist"])
