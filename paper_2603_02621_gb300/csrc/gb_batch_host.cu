@@ -276,6 +276,7 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
         cv.item_range = d_c_range;
         cv.item_chunk = d_c_chunk;
         cv.n_items = d_counts + 1;
+        cv.n_items_host = n_cover;
         cv.head = heads + 1;
         cv.Q = ctx->bq.as<uint64_t>();
         ctx->prof_begin(kProfCover, qwords * 64);

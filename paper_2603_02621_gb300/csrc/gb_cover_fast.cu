@@ -642,11 +642,11 @@ struct CoverShared {
 // One chunk of coverage words [w_begin, w_end) (32-bit words of the window a.Q,
 // 32 even n each) whose first n is n0, all in segment (row) seg, where it has
 // index j_cta.  Qc is the window's word w_begin, of which words below q_lim may
-// be read.  Called by every thread of the CTA.
+// be read.  The classes [v0, v1) of it.  Called by every thread of the CTA.
 template <int NT, int L0, bool SQ>
 __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* Qc, uint32_t q_lim, uint64_t n0,
                                             uint32_t seg, uint64_t w_begin, uint64_t w_end, uint32_t j_cta,
-                                            uint32_t* smem, CoverShared& sh)
+                                            uint32_t* smem, CoverShared& sh, uint32_t v0 = 0, uint32_t v1 = 3)
 {
     constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -701,14 +701,14 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
     uint32_t nsteps = 0;
     uint32_t recount = 0;                                   // per class (10 bits): 1 + last prime's index where no n was probed
 #pragma unroll 1
-    for (uint32_t v = 0; v < 3; ++v) {
+    for (uint32_t v = v0; v < v1; ++v) {
         unsigned long long best = 0;
         const uint32_t last = cover_class<NW, L0, SQ>(a, c, v, best, nsteps, wt);
         best = __shfl_sync(0xffffffffu, best, 0);           // (the probing's lane)
         if (best == 0) recount |= (last + 1) << (10 * v);
         else if (lane == 0) atomicMax(&sh.smax, best);
     }
-    if (threadIdx.x == 0 && c.preset) {
+    if (threadIdx.x == 0 && c.preset && v0 == 0) {
         // n = 4 = 2 + 2 and n = 6 = 3 + 3
         uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
         if (n0 == 4) {
@@ -796,7 +796,8 @@ __global__ void __launch_bounds__(NT, kCoverCtas) k_cover_fast(const CoverArgs a
     const uint64_t lim = q_words - w_begin;
     cover_chunk<NT, L0, false>(a, reinterpret_cast<const uint32_t*>(a.Q) + w_begin,
                                lim < 0xffffffffull ? (uint32_t)lim : 0xffffffffu, a.A0 + 64 * w_begin, seg, w_begin, w_end,
-                               (uint32_t)(32 * (w_begin - seg_w0)), smem, sh);
+                               (uint32_t)(32 * (w_begin - seg_w0)), smem, sh, gridDim.y == 3 ? blockIdx.y : 0,
+                               gridDim.y == 3 ? blockIdx.y + 1 : 3);
 }
 
 // Sieve and cover fused per CTA: the CTA sieves the q bits its chunk of
@@ -886,7 +887,7 @@ __global__ void __launch_bounds__(NT, kCoverCtas) k_cover_items(const CoverItems
     for (;;) {
         if (threadIdx.x == 0) s_item = atomicAdd(a.head, 1u);
         __syncthreads();
-        const uint32_t item = s_item;
+        const uint32_t part = s_item, item = part / a.split, v = part - item * a.split;
         __syncthreads();
         if (item >= n_items) break;
         const uint32_t ri = a.item_range[item];
@@ -900,7 +901,7 @@ __global__ void __launch_bounds__(NT, kCoverCtas) k_cover_items(const CoverItems
         const uint64_t lim = r.nbits / 32 - w_begin;
         cover_chunk<NT, L0, false>(c, reinterpret_cast<const uint32_t*>(a.Q + r.q_off) + w_begin,
                                    lim < 0xffffffffull ? (uint32_t)lim : 0xffffffffu, r.lo + 64 * w_begin, ri, w_begin,
-                                   w_end, (uint32_t)(32 * w_begin), smem, sh);
+                                   w_end, (uint32_t)(32 * w_begin), smem, sh, v, a.split == 3 ? v + 1 : 3);
     }
 }
 
@@ -921,6 +922,7 @@ static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
 cudaError_t launch_cover_items(const CoverItemsArgs& a0, int KA, cudaStream_t s)
 {
     CoverItemsArgs a = a0;
+    a.split = 3ull * a.n_items_host <= (uint64_t)kCoverCtas * device_sms() ? 3u : 1u;     // (as launch_l0)
     switch (cover_schedule(a.base, KA, kCoverNT / 32)) {
     case 24: return launch_items_l0<24>(a, s);
     case 32: return launch_items_l0<32>(a, s);
@@ -942,13 +944,22 @@ template <int L0>
 static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
 {
     constexpr int NT = kCoverNT;
-    const unsigned grid = a.nseg * a.chunks_per_seg;
+    unsigned grid = a.nseg * a.chunks_per_seg;
     if (grid == 0) return cudaSuccess;
     const size_t smem = CoverSmem{stream_words(a.cta_words), a.halo_words}.bytes(NT / 32);
     auto k = k_cover_fast<NT, L0>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, NT, smem, s>>>(a);
+    // one segment: only the chunks that hold some n
+    if (a.nseg == 1) {
+        const uint64_t have = ((a.n_count + 31) / 32 + a.cta_words - 1) / a.cta_words;
+        if (have < grid) grid = (unsigned)have;
+    }
+    // a call of few chunks gives each class a CTA of its own: the chunk's time is a
+    // warp's way through the classes' blocks and probings (2^16 n near 1e15: 22 ->
+    // 12 us)
+    const bool few = 3ull * grid <= (uint64_t)kCoverCtas * device_sms();
+    k<<<dim3(grid, few ? 3u : 1u), NT, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -410,6 +410,8 @@ struct CoverItemsArgs {
     const uint32_t* n_items;
     unsigned int* head;
     const uint64_t* Q;          // batch buffer
+    uint64_t n_items_host;      // the same count, on the host
+    uint32_t split;             // set by the launcher: 3 = a class of an item per CTA, else 1
 };
 cudaError_t launch_cover_items(const CoverItemsArgs& a, int KA, cudaStream_t s);
 
