@@ -166,32 +166,29 @@ uint32_t cover_generic_words(uint64_t words, uint64_t seg_words)
     return (uint32_t)std::min<uint64_t>(std::min<uint64_t>(2048, seg_words), std::max<uint64_t>(want, 256));
 }
 
+// (all that a CTA may have, 227 KB, less the kernel's static word)
+constexpr size_t kCoverSmemMax = 227 * 1024 - sizeof(unsigned long long);
+
+template <int NT>
+static cudaError_t launch_cover_nt(const CoverArgs& a, unsigned grid, cudaStream_t s)
+{
+    const size_t smem = (size_t)(2 * a.K + 1) * 4;
+    auto k = k_cover<NT>;
+    const cudaError_t e = allow_shared(k, kCoverSmemMax);
+    if (e != cudaSuccess) return e;
+    k<<<grid, NT, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_cover(const CoverArgs& a, int threads, cudaStream_t s)
 {
     const unsigned grid = a.nseg * a.chunks_per_seg;
     if (grid == 0) return cudaSuccess;
-    const size_t smem = (size_t)(2 * a.K + 1) * 4;
     switch (threads) {
-    case 128: {
-        auto k = k_cover<128>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, 128, smem, s>>>(a);
-        break;
+    case 128: return launch_cover_nt<128>(a, grid, s);
+    case 512: return launch_cover_nt<512>(a, grid, s);
+    default: return launch_cover_nt<256>(a, grid, s);
     }
-    case 512: {
-        auto k = k_cover<512>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, 512, smem, s>>>(a);
-        break;
-    }
-    default: {
-        auto k = k_cover<256>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<grid, 256, smem, s>>>(a);
-        break;
-    }
-    }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -623,14 +623,27 @@ __device__ __forceinline__ unsigned long long recount_max(const CoverArgs& a, co
 struct CoverSmem {
     uint32_t stream;            // words per stream, at most
     uint32_t halo;              // merged words below a chunk's first
-    __host__ __device__ uint32_t merged() const { return (stream + halo + 2 + 3) & ~3u; }
-    __host__ __device__ uint32_t cap(int NW) const { return (stream + 96 * NW - 1) / (96 * NW) * 96; }
-    __host__ __device__ uint32_t bytes(int NW) const { return 8 * merged() + (uint32_t)NW * cap(NW) * 6; }
+    __host__ __device__ constexpr uint32_t merged() const { return (stream + halo + 2 + 3) & ~3u; }
+    __host__ __device__ constexpr uint32_t cap(int NW) const { return (stream + 96 * NW - 1) / (96 * NW) * 96; }
+    __host__ __device__ constexpr uint32_t bytes(int NW) const { return 8 * merged() + (uint32_t)NW * cap(NW) * 6; }
 };
-__host__ __device__ __forceinline__ uint32_t stream_words(uint32_t words)
+__host__ __device__ constexpr uint32_t stream_words(uint32_t words)
 {
     const uint32_t o = (words + 2) / 3;
     return o % 3 == 0 ? o + 1 : o;
+}
+// the most dynamic shared memory a CTA is launched with: the longest chunk, the
+// longest halo (what the launchers allow, whatever the call's own size)
+constexpr uint32_t max_halo()
+{
+    int c = 0;
+    for (int v = 0; v < 3; ++v)
+        if (use_c(v, kMaxUseful - 1) > c) c = use_c(v, kMaxUseful - 1);
+    return (uint32_t)c;
+}
+constexpr uint32_t max_cover_bytes(int NT, uint32_t rounds)
+{
+    return CoverSmem{stream_words(3 * (3 * (uint32_t)NT * rounds - 1)), max_halo()}.bytes(NT / 32);
 }
 
 // shared counters of a CTA
@@ -849,10 +862,10 @@ static cudaError_t launch_seg_l0(const CoverArgs& a, const SieveArgs& sv, uint32
     const unsigned grid = a.nseg * a.chunks_per_seg;
     if (grid == 0) return cudaSuccess;
     const CoverSmem lay{stream_words(a.cta_words), a.halo_words};
-    const size_t smem = (((size_t)lay.bytes(NT / 32) / 4 + 3) & ~size_t(3)) * 4 + ((kWheelWords + 3 + 3) & ~3u) * 4 +
-                        kFusedTileBits / 8;
+    constexpr size_t rest = ((kWheelWords + 3 + 3) & ~3u) * 4 + kFusedTileBits / 8;
+    const size_t smem = (((size_t)lay.bytes(NT / 32) / 4 + 3) & ~size_t(3)) * 4 + rest;
     auto k = k_seg_cover<NT, L0>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k, ((max_cover_bytes(NT, kFusedRounds) + 15) & ~size_t(15)) + rest);
     if (e != cudaSuccess) return e;
     k<<<grid, NT, smem, s>>>(a, sv, off_w);
     return cudaGetLastError();
@@ -911,7 +924,7 @@ static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
     constexpr int NT = kCoverNT;
     const size_t smem = CoverSmem{stream_words(a.base.cta_words), a.base.halo_words}.bytes(NT / 32);
     auto k = k_cover_items<NT, L0>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k, max_cover_bytes(NT, kRounds));
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem)) != cudaSuccess) return e;
@@ -948,7 +961,7 @@ static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
     if (grid == 0) return cudaSuccess;
     const size_t smem = CoverSmem{stream_words(a.cta_words), a.halo_words}.bytes(NT / 32);
     auto k = k_cover_fast<NT, L0>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k, max_cover_bytes(NT, kRounds));
     if (e != cudaSuccess) return e;
     // one segment: only the chunks that hold some n
     if (a.nseg == 1) {

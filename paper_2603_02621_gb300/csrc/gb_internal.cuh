@@ -72,6 +72,18 @@ void fault_from_env();
 // kernels are sized as multiples of it.  1 if the query fails.
 uint32_t device_sms();
 
+// Allow launches of a kernel with up to `most` bytes of dynamic shared memory.
+// The limit belongs to the kernel on the device, not to a launch: with host
+// threads of several contexts in the same launcher, one that set it to its own
+// call's size would lower it between another's set and launch.  So a launcher
+// passes the most it ever launches the kernel with, the same on every call, and
+// its own size to the launch alone.
+template <class K>
+cudaError_t allow_shared(K* kernel, size_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Barrett reduction (P. Barrett, CRYPTO '86): with m = floor((2^64-1)/p), the
 // quotient estimate hi64(x*m) is at most 2 below floor(x/p); two conditional
 // subtractions finish the remainder.  p < 2^32, any 64-bit x.

@@ -144,12 +144,15 @@ __global__ void __launch_bounds__(NT) k_sieve_items(const SieveItemsArgs a)
     }
 }
 
+// of the longest tile (gb_config::tile_bits is at most 2^20)
+constexpr size_t kSieveSmemMax = (kWheelWords + 3) * 4 + (1u << 20) / 8;
+
 template <int NT>
 static cudaError_t launch_sieve_items_nt(const SieveItemsArgs& a, cudaStream_t s)
 {
     const size_t smem = (kWheelWords + 3) * 4 + (size_t)a.base.tile_bits / 8;
     auto k = k_sieve_items<NT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_shared(k, kSieveSmemMax);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, NT, smem)) != cudaSuccess) return e;
@@ -167,38 +170,27 @@ cudaError_t launch_sieve_items(const SieveItemsArgs& a, int threads, cudaStream_
     }
 }
 
+template <int NT>
+static cudaError_t launch_sieve_nt(const SieveArgs& a, cudaStream_t s)
+{
+    const uint64_t tiles = (a.nbits + a.tile_bits - 1) / a.tile_bits;
+    const size_t smem = (kWheelWords + 3) * 4 + (size_t)a.tile_bits / 8;
+    auto k = k_sieve<NT>;
+    const cudaError_t e = allow_shared(k, kSieveSmemMax);
+    if (e != cudaSuccess) return e;
+    k<<<(unsigned)tiles, NT, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sieve(const SieveArgs& a, int threads, cudaStream_t s)
 {
     if (a.nbits == 0) return cudaSuccess;
-    const uint64_t tiles = (a.nbits + a.tile_bits - 1) / a.tile_bits;
-    const size_t smem = (kWheelWords + 3) * 4 + (size_t)a.tile_bits / 8;
     switch (threads) {
-    case 128: {
-        auto k = k_sieve<128>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<(unsigned)tiles, 128, smem, s>>>(a);
-        break;
+    case 128: return launch_sieve_nt<128>(a, s);
+    case 512: return launch_sieve_nt<512>(a, s);
+    case 1024: return launch_sieve_nt<1024>(a, s);
+    default: return launch_sieve_nt<256>(a, s);
     }
-    case 512: {
-        auto k = k_sieve<512>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<(unsigned)tiles, 512, smem, s>>>(a);
-        break;
-    }
-    case 1024: {
-        auto k = k_sieve<1024>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<(unsigned)tiles, 1024, smem, s>>>(a);
-        break;
-    }
-    default: {
-        auto k = k_sieve<256>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k<<<(unsigned)tiles, 256, smem, s>>>(a);
-        break;
-    }
-    }
-    return cudaGetLastError();
 }
 
 // slice primes below this take the mod-30 wheel (their strikes per slice,
