@@ -166,8 +166,8 @@ uint32_t cover_generic_words(uint64_t words, uint64_t seg_words)
     return (uint32_t)std::min<uint64_t>(std::min<uint64_t>(2048, seg_words), std::max<uint64_t>(want, 256));
 }
 
-// (all that a CTA may have, 227 KB, less the kernel's static word)
-constexpr size_t kCoverSmemMax = 227 * 1024 - sizeof(unsigned long long);
+// (all that a CTA may have, 227 KB, less the kernel's 16 static bytes)
+constexpr size_t kCoverSmemMax = 227 * 1024 - 16;
 
 template <int NT>
 static cudaError_t launch_cover_nt(const CoverArgs& a, unsigned grid, cudaStream_t s)

@@ -81,7 +81,9 @@ uint32_t device_sms();
 template <class K>
 cudaError_t allow_shared(K* kernel, size_t most)
 {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) cudaGetLastError();               // (not the next launch's error)
+    return e;
 }
 
 // Barrett reduction (P. Barrett, CRYPTO '86): with m = floor((2^64-1)/p), the

@@ -50,11 +50,12 @@ def _same(a, b):
 @pytest.mark.parametrize("kind", ["range", "batch", "pmin", "sieve"])
 def test_small_and_large_calls_at_once(gbm, kind):
     with gbm.Context(device=0, base_limit=1 << 21, p1=1 << 15, p2=0) as parent:
-        streams = [torch.cuda.Stream() for _ in range(2)]
+        size = [False] * 4 + [True]
+        streams = [torch.cuda.Stream() for _ in size]
         ctxs = [parent.share(s.cuda_stream) for s in streams]
-        calls = [_calls(gbm, kind, large) for large in (False, True)]
+        calls = [_calls(gbm, kind, large) for large in size]
         want = [f(g) for f, g in zip(calls, ctxs)]
-        stop, errors, done = threading.Event(), [], [0, 0]
+        stop, errors, done = threading.Event(), [], [0] * len(size)
 
         def loop(i, most):
             try:
@@ -67,7 +68,7 @@ def test_small_and_large_calls_at_once(gbm, kind):
                 errors.append(e)
             stop.set()                              # the small calls go on for as long as the large ones
 
-        threads = [threading.Thread(target=loop, args=a) for a in ((0, 10**6), (1, 400))]
+        threads = [threading.Thread(target=loop, args=(i, 1500 if large else 10**6)) for i, large in enumerate(size)]
         for t in threads:
             t.start()
         for t in threads:
@@ -75,4 +76,4 @@ def test_small_and_large_calls_at_once(gbm, kind):
         for g in ctxs:
             g.close()
     assert not errors, errors
-    assert done[0] > 0 and done[1] == 400
+    assert min(done) > 0 and done[-1] == 1500
