@@ -204,7 +204,7 @@ extern "C" int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, ui
         ra.pmin = out->pmin;
         ra.items = items;
         ra.count = counters;
-        ra.cap = (uint32_t)n_words;                          // one item per word at most: never full
+        ra.cap = (uint32_t)n_words;
         NA_CUDA(gb::launch_retry(ra, s));
     }
     const uint32_t row_stride = want_rows ? out->seg_hist_stride : 0;
@@ -230,6 +230,7 @@ extern "C" int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, ui
     fa.records = out->segs ? (segs_dev ? reinterpret_cast<gb::SegRecord*>(out->segs) : records) : nullptr;
     fa.nrecords = out->segs && out->seg_cap ? 1u : 0u;
     fa.totals = totals;
+    fa.retry_count = retry ? counters : nullptr;
     NA_CUDA(gb::launch_finalize(fa, s));
 
     gb::RangeTotals tot{};
@@ -241,6 +242,10 @@ extern "C" int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, ui
     if (want_rows && !rows_dev)
         NA_CUDA(cudaMemcpyAsync(out->seg_hist, rows, (size_t)row_stride * 8, cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
+    // The block cover files an item per open n, up to 64 for a word, and the list
+    // holds one per word (the generic cover's items): where a small P1 leaves more
+    // n open, the call is done over in one pass to Pf, which has no retry list.
+    if (retry && tot.open > n_words) return gb_verify_range_noalloc(ctx, lo, hi, Pf, out);
     if (out->hist)
         for (uint32_t i = nh; i < out->hist_cap; ++i) out->hist[i] = 0;
     out->n_checked = n_total;
