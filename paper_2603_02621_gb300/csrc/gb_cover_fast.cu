@@ -43,8 +43,8 @@
 // from the probing when any n reached it: every n of the class covered by the
 // blocks has a smaller one.  Where a later block covers all that was open, its
 // input list is still there and is run once more, recording it; where block 0
-// does (a few words only), the words are, unless block 0's last prime is below
-// the chunk's maximum so far.
+// does (a few words only), or no probed n is covered (a small bound), the merged
+// words are, unless the blocks' last prime is below the chunk's maximum so far.
 //
 // Bound: the ALU pipe and the popcounts of block 0 (a step on three words is 8
 // ALU, 2 popcount and 3 multiply-add instructions).  2^32 n from 4 on, 2^33
@@ -467,6 +467,31 @@ __device__ __forceinline__ void probe_warp(const CoverArgs& a, const Chunk& c, u
     }
 }
 
+// The key of the largest p_min, with its smallest n, that the useful primes I0 ..
+// I1 - 1 give the n open in merged word k of class v (C: its coverage before them;
+// 0: none).  From the merged words in shared memory, every lane a word of its own.
+__device__ __forceinline__ unsigned long long track_word(const Chunk& c, uint32_t v, uint32_t k, uint32_t C, uint32_t I0,
+                                                         uint32_t I1)
+{
+    const uint32_t f = n_phase(c, v, k);
+    uint32_t last = 0, bits = 0;
+    for (uint32_t i = I0; i < I1 && C != 0xffffffffu; ++i) {
+        const uint32_t p = kClassDev.p[v][i], d = (p - 3) >> 1, w = (d + 31) >> 5;
+        const uint32_t* y = ((v + 3 - p % 3) % 3 == 1 ? c.Y1 : c.Y2) + k - w;
+        const uint32_t nw = ((d & 31) ? __funnelshift_r(y[0], y[1], 32 - (d & 31)) : y[0]) & ~C;
+        C |= nw;
+        if (nw) {
+            last = i + 1;
+            bits = nw;
+        }
+    }
+    if (!last) return 0;
+    // the smallest n of the bits: of each stream's lowest
+    uint32_t n = 0xffffffffu;
+    for (uint32_t m = bits; m; m &= m - 1) n = min(n, merged_n(c, f, k, __ffs(m) - 1));
+    return ((unsigned long long)(kClassDev.k[v][last - 1] + 2) << 32) | (0xffffffffull - (c.j_cta + n));
+}
+
 // The largest p_min, with its smallest n, that the block of kLater useful primes
 // from I0 on gives the n open in the list (which it covers entirely, so that the
 // list is still there as it was before).
@@ -474,33 +499,31 @@ __device__ __forceinline__ unsigned long long track_block(const Chunk& c, uint32
 {
     unsigned long long best = 0;
     for (uint32_t e = threadIdx.x & 31; e < n_in; e += 32) {
-        const uint32_t k = c.lw[e], f = n_phase(c, v, k);
-        uint32_t C = c.lc[e], last = 0, bits = 0;
-        for (uint32_t i = 0; i < (uint32_t)kLater; ++i) {
-            const uint32_t p = kClassDev.p[v][I0 + i], d = (p - 3) >> 1, w = (d + 31) >> 5;
-            const uint32_t* y = ((v + 3 - p % 3) % 3 == 1 ? c.Y1 : c.Y2) + k - w;
-            const uint32_t nw = ((d & 31) ? __funnelshift_r(y[0], y[1], 32 - (d & 31)) : y[0]) & ~C;
-            C |= nw;
-            if (nw) {
-                last = i + 1;
-                bits = nw;
-            }
-        }
-        if (!last) continue;
-        // the smallest n of the bits: of each stream's lowest
-        uint32_t n = 0xffffffffu;
-        for (uint32_t m = bits; m; m &= m - 1) n = min(n, merged_n(c, f, k, __ffs(m) - 1));
-        const unsigned long long key =
-            ((unsigned long long)(kClassDev.k[v][I0 + last - 1] + 2) << 32) | (0xffffffffull - (c.j_cta + n));
+        const unsigned long long key = track_word(c, v, c.lw[e], c.lc[e], I0, I0 + kLater);
         if (key > best) best = key;
     }
     return warp_max_key(best);
 }
 
+// The largest p_min among the first L useful primes, with its smallest n, of all
+// the warp's merged words of class v.
+template <int NW>
+__device__ __forceinline__ unsigned long long track_all(const Chunk& c, uint32_t v, uint32_t L)
+{
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long best = 0;
+    for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW)
+        for (uint32_t k = wbase + lane; k < wbase + 96 && k < c.O; k += 32) {
+            const unsigned long long key = track_word(c, v, k, init_c(c, v, k), 0, L);
+            if (key > best) best = key;
+        }
+    return warp_max_key(best);
+}
+
 // Class v of a chunk: block 0 over the warp's merged words, the later blocks
 // over its open ones, probing.  best: the largest key of what block 0 left open
-// (0: none of that was covered); returns the odd-prime index of the blocks' last prime (an upper bound of the
-// others' p_min).
+// (0: none of that was covered); returns the number of useful primes in the blocks
+// run (the last of them bounds the others' p_min).
 template <int NW, int L0, bool SQ>
 __device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk& c, uint32_t v,
                                                 unsigned long long& best, uint32_t& nsteps, const uint32_t (&wt)[3])
@@ -585,37 +608,10 @@ __device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk&
         if (n_out == 0) best = track_block(c, v, n_open, L0 + kLater * (b - 1));
         n_open = n_out;
     }
-    const uint32_t last = kClassDev.k[v][L0 + kLater * (b - 1) - 1];
-    probe_warp<SQ>(a, c, v, n_open, last + 1, best, nsteps);
+    const uint32_t used = (uint32_t)(L0 + kLater * (b - 1));
+    probe_warp<SQ>(a, c, v, n_open, kClassDev.k[v][used - 1] + 1u, best, nsteps);
     __syncwarp();                                           // the list is the next class's
-    return last;
-}
-
-// The largest p_min among the first k_end + 1 odd primes, with its smallest n, of
-// the warp's words of class v: the plain words once more, one per lane.
-template <int NW, bool SQ>
-__device__ __forceinline__ unsigned long long recount_max(const CoverArgs& a, const Chunk& c, uint32_t v, uint32_t k_end)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long best = 0;
-    for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW)
-        for (uint32_t i = 0; i < 9; ++i) {
-            const uint32_t k = wbase + 32 * (i % 3) + lane, W = k + (i / 3) * c.O;
-            uint32_t open = k < c.O ? valid_bits(c, W) & phase_mask(n_phase(c, v, W)) : 0u;
-            for (uint32_t kk = 0; kk <= k_end && __any_sync(0xffffffffu, open != 0); ++kk) {
-                if (!open) continue;
-                const uint32_t d = (a.H - __ldg(a.primes + 1 + kk) - 1) >> 1;
-                const uint32_t* q = c.Qc + W + (d >> 5);
-                const uint32_t nw = ((d & 31) ? __funnelshift_r(ldq<SQ>(q), ldq<SQ>(q + 1), d & 31) : ldq<SQ>(q)) & open;
-                open &= ~nw;
-                if (nw) {
-                    const uint32_t j = c.j_cta + 32 * W + (__ffs(nw) - 1);
-                    const unsigned long long key = ((unsigned long long)(kk + 2) << 32) | (0xffffffffull - j);
-                    if (key > best) best = key;
-                }
-            }
-        }
-    return warp_max_key(best);
+    return used;
 }
 
 // dynamic shared memory of a CTA: the merged words of both residues, then the
@@ -712,13 +708,13 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
     __syncthreads();
 
     uint32_t nsteps = 0;
-    uint32_t recount = 0;                                   // per class (10 bits): 1 + last prime's index where no n was probed
+    uint32_t recount = 0;                                   // per class (8 bits): useful primes of the blocks where no probed n was covered
 #pragma unroll 1
     for (uint32_t v = v0; v < v1; ++v) {
         unsigned long long best = 0;
-        const uint32_t last = cover_class<NW, L0, SQ>(a, c, v, best, nsteps, wt);
+        const uint32_t used = cover_class<NW, L0, SQ>(a, c, v, best, nsteps, wt);
         best = __shfl_sync(0xffffffffu, best, 0);           // (the probing's lane)
-        if (best == 0) recount |= (last + 1) << (10 * v);
+        if (best == 0) recount |= used << (8 * v);
         else if (lane == 0) atomicMax(&sh.smax, best);
     }
     if (threadIdx.x == 0 && c.preset && v0 == 0) {
@@ -735,13 +731,15 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
         }
     }
     __syncthreads();
-    // classes of which no n was probed: the maximum lies in the blocks
+    // classes of which no probed n was covered: the maximum lies in the blocks.  From
+    // the merged words in shared memory (10^4 n near 1e15 with the bound 1024: 30 us;
+    // from the window's words in global memory, a load's latency per prime, 176)
 #pragma unroll 1
     for (uint32_t v = 0; v < 3 && recount; ++v) {
-        const uint32_t last1 = (recount >> (10 * v)) & 1023u;
+        const uint32_t used = (recount >> (8 * v)) & 255u;
         const uint32_t top = (uint32_t)(*(volatile unsigned long long*)&sh.smax >> 32);
-        if (__any_sync(0xffffffffu, last1 && last1 + 1 >= top)) {
-            const unsigned long long key = recount_max<NW, SQ>(a, c, v, last1 - 1);
+        if (__any_sync(0xffffffffu, used && kClassDev.k[v][used ? used - 1 : 0] + 2u >= top)) {
+            const unsigned long long key = track_all<NW>(c, v, used);
             if (lane == 0 && key) atomicMax(&sh.smax, key);
         }
     }
