@@ -86,6 +86,12 @@ constexpr uint32_t kProbeWords = 3;
 // too small to give every SM its chunks.
 constexpr int kCoverNT = 512, kFusedNT = 256;
 constexpr int kCoverCtas = 2;                               // per SM
+// Chunks of at most 96 merged words (segments of 2^11 .. 2^13) are one warp per
+// class: CTAs of 128, eight per SM.  2^24 n near 1e12, segments of 2^11, 2^12 and
+// 2^13: 72, 39 and 25 us (319, 166 and 98 with CTAs of 512 whose first warp took
+// the three classes one after the other).
+constexpr int kShortNT = 128;
+constexpr uint32_t kShortStream = 96;
 constexpr uint32_t kRounds = 5;
 constexpr uint32_t kFusedRounds = 3;                        // (the fused tile holds no more)
 static_assert(kRounds <= kMaxRounds, "10-bit counters");
@@ -316,6 +322,7 @@ struct Chunk {
     uint32_t preset;            // bits of word 0: n = 4 and n = 6
     uint64_t w_begin;           // the chunk's first word in the slab
     uint32_t j_cta, seg;
+    uint32_t k_first;           // this warp's first merged word (then every 96 NW words on)
     uint32_t* lc;               // this warp's list: coverage, merged word index
     uint16_t* lw;
     uint32_t* shist;            // the CTA's bins [3][kMaxUseful]
@@ -510,9 +517,9 @@ __device__ __forceinline__ unsigned long long track_block(const Chunk& c, uint32
 template <int NW>
 __device__ __forceinline__ unsigned long long track_all(const Chunk& c, uint32_t v, uint32_t L)
 {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31;
     unsigned long long best = 0;
-    for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW)
+    for (uint32_t wbase = c.k_first; wbase < c.O; wbase += 96 * NW)
         for (uint32_t k = wbase + lane; k < wbase + 96 && k < c.O; k += 32) {
             const unsigned long long key = track_word(c, v, k, init_c(c, v, k), 0, L);
             if (key > best) best = key;
@@ -528,7 +535,7 @@ template <int NW, int L0, bool SQ>
 __device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk& c, uint32_t v,
                                                 unsigned long long& best, uint32_t& nsteps, const uint32_t (&wt)[3])
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     uint32_t n_open = 0;
     uint32_t* const bins = c.shist + v * kMaxUseful;
     {
@@ -537,7 +544,7 @@ __device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk&
 #pragma unroll
         for (int k = 0; k < KH; ++k) cum[k] = 0;
         uint32_t init_pop = 0;
-        for (uint32_t wbase = 96 * warp; wbase < c.O; wbase += 96 * NW) {
+        for (uint32_t wbase = c.k_first; wbase < c.O; wbase += 96 * NW) {
             const uint32_t wl = wbase + 3 * (uint32_t)lane;           // the lane's first word
             uint32_t C0 = 0, C1 = 0, C2 = 0;
             if (wl + 2 >= c.O || 32 * (wl + 3 + 2 * c.O) > c.n_end || (wl == 0 && c.preset)) {
@@ -709,6 +716,19 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
 
     uint32_t nsteps = 0;
     uint32_t recount = 0;                                   // per class (8 bits): useful primes of the blocks where no probed n was covered
+    // In a short chunk most warps would have no words, and the others the three classes
+    // one after the other: there each class has warps of its own (2^24 n near 1e12 in
+    // segments of 2^14: 59 -> 35 us).
+    c.k_first = 96 * (uint32_t)warp;
+    const uint32_t busy = (c.O + 95) / 96;
+    if (v1 - v0 == 3 && 3 * busy <= (uint32_t)NW) {
+        const uint32_t own = (uint32_t)warp / busy;
+        c.k_first -= 96 * busy * own;
+        v0 = own;
+        v1 = own < 3 ? own + 1 : own;
+    } else if (c.k_first >= c.O) {
+        v1 = v0;
+    }
 #pragma unroll 1
     for (uint32_t v = v0; v < v1; ++v) {
         unsigned long long best = 0;
@@ -717,7 +737,7 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
         if (best == 0) recount |= used << (8 * v);
         else if (lane == 0) atomicMax(&sh.smax, best);
     }
-    if (threadIdx.x == 0 && c.preset && v0 == 0) {
+    if (threadIdx.x == 0 && c.preset && v0 == 0) {          // (thread 0 has the first class of a whole chunk)
         // n = 4 = 2 + 2 and n = 6 = 3 + 3
         uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
         if (n0 == 4) {
@@ -788,7 +808,7 @@ static int cover_schedule(CoverArgs& a, int KA, int NW)
 }
 
 template <int NT, int L0>
-__global__ void __launch_bounds__(NT, kCoverCtas) k_cover_fast(const CoverArgs a)
+__global__ void __launch_bounds__(NT, kCoverCtas * kCoverNT / NT) k_cover_fast(const CoverArgs a)
 {
     extern __shared__ uint32_t smem[];
     __shared__ CoverShared sh;
@@ -951,10 +971,9 @@ int cover_fast_phase_primes(uint32_t K, uint64_t n_hi)
     return ka >= 48 ? ka : 0;
 }
 
-template <int L0>
-static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
+template <int NT, int L0>
+static cudaError_t launch_nt(const CoverArgs& a, cudaStream_t s)
 {
-    constexpr int NT = kCoverNT;
     unsigned grid = a.nseg * a.chunks_per_seg;
     if (grid == 0) return cudaSuccess;
     const size_t smem = CoverSmem{stream_words(a.cta_words), a.halo_words}.bytes(NT / 32);
@@ -972,6 +991,12 @@ static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
     const bool few = 3ull * grid <= (uint64_t)kCoverCtas * device_sms();
     k<<<dim3(grid, few ? 3u : 1u), NT, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+template <int L0>
+static cudaError_t launch_l0(const CoverArgs& a, cudaStream_t s)
+{
+    return stream_words(a.cta_words) <= kShortStream ? launch_nt<kShortNT, L0>(a, s) : launch_nt<kCoverNT, L0>(a, s);
 }
 
 cudaError_t launch_cover_fast(const CoverArgs& a0, int KA, cudaStream_t s)
