@@ -91,6 +91,7 @@ constexpr int kCoverCtas = 2;                               // per SM
 // 2^13: 72, 39 and 25 us (319, 166 and 98 with CTAs of 512 whose first warp took
 // the three classes one after the other).
 constexpr int kShortNT = 128;
+constexpr int kMaxWarps = kCoverNT / 32;
 constexpr uint32_t kShortStream = 96;
 constexpr uint32_t kRounds = 5;
 constexpr uint32_t kFusedRounds = 3;                        // (the fused tile holds no more)
@@ -512,21 +513,6 @@ __device__ __forceinline__ unsigned long long track_block(const Chunk& c, uint32
     return warp_max_key(best);
 }
 
-// The largest p_min among the first L useful primes, with its smallest n, of all
-// the warp's merged words of class v.
-template <int NW>
-__device__ __forceinline__ unsigned long long track_all(const Chunk& c, uint32_t v, uint32_t L)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    unsigned long long best = 0;
-    for (uint32_t wbase = c.k_first; wbase < c.O; wbase += 96 * NW)
-        for (uint32_t k = wbase + lane; k < wbase + 96 && k < c.O; k += 32) {
-            const unsigned long long key = track_word(c, v, k, init_c(c, v, k), 0, L);
-            if (key > best) best = key;
-        }
-    return warp_max_key(best);
-}
-
 // Class v of a chunk: block 0 over the warp's merged words, the later blocks
 // over its open ones, probing.  best: the largest key of what block 0 left open
 // (0: none of that was covered); returns the number of useful primes in the blocks
@@ -653,6 +639,8 @@ constexpr uint32_t max_cover_bytes(int NT, uint32_t rounds)
 struct CoverShared {
     uint32_t hist[3 * kMaxUseful];
     unsigned long long smax;
+    uint32_t any;               // 1: some of these
+    uint8_t used[3][kMaxWarps]; // per class and warp (by its words) whose probing covered nothing: cover_class's value
 };
 
 // One chunk of coverage words [w_begin, w_end) (32-bit words of the window a.Q,
@@ -692,7 +680,11 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
 
     __syncthreads();                                        // shared memory free (previous chunk)
     for (uint32_t k = threadIdx.x; k < 3 * kMaxUseful; k += NT) sh.hist[k] = 0;
-    if (threadIdx.x == 0) sh.smax = 0;
+    if (threadIdx.x == 0) {
+        sh.smax = 0;
+        sh.any = 0;
+    }
+    if (threadIdx.x < 3 * kMaxWarps) (&sh.used[0][0])[threadIdx.x] = 0;
     {
         // merged words: the window words of the three streams, from halo words
         // below the first coverage word's partner of p = 3 on; q = Bc + 2 (32 W + b)
@@ -715,7 +707,6 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
     __syncthreads();
 
     uint32_t nsteps = 0;
-    uint32_t recount = 0;                                   // per class (8 bits): useful primes of the blocks where no probed n was covered
     // In a short chunk most warps would have no words, and the others the three classes
     // one after the other: there each class has warps of its own (2^24 n near 1e12 in
     // segments of 2^14: 59 -> 35 us).
@@ -734,8 +725,14 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
         unsigned long long best = 0;
         const uint32_t used = cover_class<NW, L0, SQ>(a, c, v, best, nsteps, wt);
         best = __shfl_sync(0xffffffffu, best, 0);           // (the probing's lane)
-        if (best == 0) recount |= used << (8 * v);
-        else if (lane == 0) atomicMax(&sh.smax, best);
+        if (lane == 0) {
+            if (best) {
+                atomicMax(&sh.smax, best);
+            } else {
+                sh.used[v][c.k_first / 96] = (uint8_t)used;
+                sh.any = 1;
+            }
+        }
     }
     if (threadIdx.x == 0 && c.preset && v0 == 0) {          // (thread 0 has the first class of a whole chunk)
         // n = 4 = 2 + 2 and n = 6 = 3 + 3
@@ -751,15 +748,33 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
         }
     }
     __syncthreads();
-    // classes of which no probed n was covered: the maximum lies in the blocks.  From
-    // the merged words in shared memory (10^4 n near 1e15 with the bound 1024: 30 us;
-    // from the window's words in global memory, a load's latency per prime, 176)
+    // Warps and classes of which no probed n was covered: the maximum lies in the
+    // blocks.  Where it may be the chunk's and the segment's, the whole CTA goes
+    // through their merged words once more (10^4 n near 1e15 with the bound 1024:
+    // 18 us; 30 by the warp itself, 176 from the window's words in global memory, a
+    // load's latency per prime).
+    if (sh.any) {
 #pragma unroll 1
-    for (uint32_t v = 0; v < 3 && recount; ++v) {
-        const uint32_t used = (recount >> (8 * v)) & 255u;
-        const uint32_t top = (uint32_t)(*(volatile unsigned long long*)&sh.smax >> 32);
-        if (__any_sync(0xffffffffu, used && kClassDev.k[v][used ? used - 1 : 0] + 2u >= top)) {
-            const unsigned long long key = track_all<NW>(c, v, used);
+        for (uint32_t v = 0; v < 3; ++v) {
+            // the class's last prime that covered an n of the chunk, 2 + its index as in
+            // the keys, and the maximum so far
+            uint32_t last = 0;
+            for (uint32_t i = lane; i < (uint32_t)kMaxUseful; i += 32)
+                if (c.shist[v * kMaxUseful + i]) last = i + 1;
+            last = __reduce_max_sync(0xffffffffu, last);
+            const uint32_t top = max((uint32_t)(*(volatile unsigned long long*)&sh.smax >> 32),
+                                     (uint32_t)(*(volatile unsigned long long*)&a.maxkey[seg] >> 32));
+            uint32_t n = lane < kMaxWarps ? min(last, (uint32_t)sh.used[v][lane]) : 0u;
+            if (n && kClassDev.k[v][n - 1] + 2u < top) n = 0;
+            const unsigned redo = __ballot_sync(0xffffffffu, n != 0);
+            if (!redo) continue;
+            unsigned long long key = 0;
+            for (uint32_t k = threadIdx.x; k < c.O; k += NT)
+                if ((redo >> (k / 96 % NW)) & 1u) {
+                    const unsigned long long t = track_word(c, v, k, init_c(c, v, k), 0, last);
+                    if (t > key) key = t;
+                }
+            key = warp_max_key(key);
             if (lane == 0 && key) atomicMax(&sh.smax, key);
         }
     }
