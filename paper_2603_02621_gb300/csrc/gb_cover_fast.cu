@@ -768,12 +768,16 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
             if (n && kClassDev.k[v][n - 1] + 2u < top) n = 0;
             const unsigned redo = __ballot_sync(0xffffffffu, n != 0);
             if (!redo) continue;
+            // a third of a flagged warp's 96 words to each warp of the CTA
+            const uint32_t thirds = 3 * ((c.O + 96 * NW - 1) / (96 * NW));
             unsigned long long key = 0;
-            for (uint32_t k = threadIdx.x; k < c.O; k += NT)
-                if ((redo >> (k / 96 % NW)) & 1u) {
-                    const unsigned long long t = track_word(c, v, k, init_c(c, v, k), 0, last);
-                    if (t > key) key = t;
-                }
+            for (uint32_t u = warp; u < __popc(redo) * thirds; u += NW) {
+                const uint32_t slot = __fns(redo, 0, (int)(u / thirds) + 1), r = u % thirds;
+                const uint32_t k = 96 * (slot + NW * (r / 3)) + 32 * (r % 3) + lane;
+                if (k >= c.O) continue;
+                const unsigned long long t = track_word(c, v, k, init_c(c, v, k), 0, last);
+                if (t > key) key = t;
+            }
             key = warp_max_key(key);
             if (lane == 0 && key) atomicMax(&sh.smax, key);
         }
