@@ -565,8 +565,9 @@ __device__ __forceinline__ uint32_t cover_class(const CoverArgs& a, const Chunk&
     __syncwarp();
     // later blocks over the list, in batches of 32 words (one per lane); the
     // words still open move up in it (each batch is read before its outputs land)
+    const int n_later = (int)(v == 0 ? a.n_later[0] : v == 1 ? a.n_later[1] : a.n_later[2]);
     int b = 1;
-    for (; b <= (int)a.n_later && n_open > kProbeWords; ++b) {
+    for (; b <= n_later && n_open > kProbeWords; ++b) {
         constexpr int KH = (kLater + 2) / 3;
         uint32_t cum[KH];
 #pragma unroll
@@ -804,23 +805,41 @@ bool cover_prefix_valid(int KA) { return KA >= 48 && KA <= kMaxPrefix && KA % 16
 // the pass has no more than the 48 primes that hold them, 48 near 1e17 and above
 // (KA = 240), 32 otherwise (2^33 n near 5e11: 2.69 ms with 28, 2.64 with 32, 2.67
 // with 36, 2.72 with 40; 2^31 near 1e15: 0.89, 0.87, 0.86, 0.85).
+// A bound below about 900 cuts the blocks short, each class's on its own: every n that
+// they leave open is probed, 32 primes to a warp, whether or not a prime is useful to
+// it.  There the n divisible by 3, to which every prime is useful, go through KA of them,
+// and block 0 takes 24 where whole blocks after it then reach further in the other
+// classes (10^8 n near 1e12 with P = 227, 300, 512 and 700: 2.39, 1.44, 0.20 and 0.08
+// ms; 2.68, 1.78, 0.47 and 0.11 with the blocks that all three classes have room for;
+// with P = 900 near 1e15 0.090 and 0.113, from 1024 on equal).
+constexpr uint32_t kSmallK = 160;
 static int cover_schedule(CoverArgs& a, int KA, int NW)
 {
     if (!cover_prefix_valid(KA) || (uint32_t)KA > a.K || a.cta_words == 0) return 0;
     if (stream_words(a.cta_words) > kMaxRounds * 96u * (uint32_t)NW) return 0;
-    auto fits = [&](int n) {                                // the first n useful primes of each class are in the pass
-        for (int v = 0; v < 3; ++v)
-            if (kClass.k[v][n - 1] >= a.K) return false;
-        return true;
+    int room[3];                                            // useful primes of the class in the pass
+    for (int v = 0; v < 3; ++v) {
+        room[v] = 0;
+        while (room[v] < kMaxUseful && kClass.k[v][room[v]] < a.K) ++room[v];
+    }
+    const int least = std::min(room[0], std::min(room[1], room[2]));
+    const int want = KA / 2 + 8;
+    auto later = [&](int have, int L0, int to) {            // whole blocks after block 0
+        return std::max(0, std::min((to - L0 + kLater - 1) / kLater, (have - L0) / kLater));
     };
-    const int L0 = KA >= 240 && fits(48) ? 48 : fits(32) ? 32 : fits(24) ? 24 : 0;
+    int L0 = KA >= 240 && least >= 48 ? 48 : least >= 32 ? 32 : least >= 24 ? 24 : 0;
     if (!L0) return 0;
-    int later = (KA / 2 + 8 - L0 + kLater - 1) / kLater;
-    while (later > 0 && (L0 + kLater * later > kMaxUseful || !fits(L0 + kLater * later))) --later;
-    a.n_later = (uint32_t)(later > 0 ? later : 0);
+    const bool small = a.K < kSmallK &&
+                       L0 + kLater * later(std::min(room[1], room[2]), L0, want) < want;
+    if (small && L0 == 32 &&
+        later(room[1], 24, want) + later(room[2], 24, want) > later(room[1], 32, want) + later(room[2], 32, want))
+        L0 = 24;
     a.halo_words = 0;
-    for (int v = 0; v < 3; ++v)
-        a.halo_words = std::max<uint32_t>(a.halo_words, (uint32_t)use_c(v, L0 + kLater * (int)a.n_later - 1));
+    for (int v = 0; v < 3; ++v) {
+        const int n = small ? later(room[v], L0, v == 0 ? KA : want) : later(least, L0, want);
+        a.n_later[v] = (uint32_t)n;
+        a.halo_words = std::max<uint32_t>(a.halo_words, (uint32_t)use_c(v, L0 + kLater * n - 1));
+    }
     if (((a.H - 4) >> 6) < a.halo_words) return 0;
     a.cum_wt[0] = 1; a.cum_wt[1] = 1u << kCumBits; a.cum_wt[2] = 1u << (2 * kCumBits);
     return L0;

@@ -296,7 +296,7 @@ struct CoverArgs {
     int max_only;
     const unsigned long long* maxkey_check;
     // block cover only (set by the launcher)
-    uint32_t n_later;           // blocks after block 0
+    uint32_t n_later[3];        // blocks after block 0, of each class
     uint32_t halo_words;        // words below a word's partner of p = 3 that the blocks read
     uint32_t cum_wt[3];         // 1, 2^10, 2^20: weights of the packed 10-bit counters
 };
