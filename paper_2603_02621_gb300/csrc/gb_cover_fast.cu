@@ -640,6 +640,7 @@ constexpr uint32_t max_cover_bytes(int NT, uint32_t rounds)
 struct CoverShared {
     uint32_t hist[3 * kMaxUseful];
     unsigned long long smax;
+    uint32_t top;               // 2 + the index of the largest p_min known when these are gone through
     uint32_t any;               // 1: some of these
     uint8_t used[3][kMaxWarps]; // per class and warp (by its words) whose probing covered nothing: cover_class's value
 };
@@ -755,16 +756,18 @@ __device__ __forceinline__ void cover_chunk(const CoverArgs& a, const uint32_t* 
     // 18 us; 30 by the warp itself, 176 from the window's words in global memory, a
     // load's latency per prime).
     if (sh.any) {
+        // (one value for all warps, which share out the words by it)
+        if (threadIdx.x == 0)
+            sh.top = max((uint32_t)(sh.smax >> 32), (uint32_t)(*(volatile unsigned long long*)&a.maxkey[seg] >> 32));
+        __syncthreads();
+        const uint32_t top = sh.top;
 #pragma unroll 1
         for (uint32_t v = 0; v < 3; ++v) {
-            // the class's last prime that covered an n of the chunk, 2 + its index as in
-            // the keys, and the maximum so far
+            // the class's last prime that covered an n of the chunk
             uint32_t last = 0;
             for (uint32_t i = lane; i < (uint32_t)kMaxUseful; i += 32)
                 if (c.shist[v * kMaxUseful + i]) last = i + 1;
             last = __reduce_max_sync(0xffffffffu, last);
-            const uint32_t top = max((uint32_t)(*(volatile unsigned long long*)&sh.smax >> 32),
-                                     (uint32_t)(*(volatile unsigned long long*)&a.maxkey[seg] >> 32));
             uint32_t n = lane < kMaxWarps ? min(last, (uint32_t)sh.used[v][lane]) : 0u;
             if (n && kClassDev.k[v][n - 1] + 2u < top) n = 0;
             const unsigned redo = __ballot_sync(0xffffffffu, n != 0);

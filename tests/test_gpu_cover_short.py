@@ -61,3 +61,17 @@ def test_short_segments_time(gbm):
     a = _cover_ms(gbm, 10**12, 1 << 24, p1=1 << 15, seg_len=1 << 11)
     b = _cover_ms(gbm, 10**12, 1 << 24, p1=1 << 15, seg_len=1 << 16)
     assert a < 6 * b, (a, b)
+
+
+@pytest.mark.parametrize("lo,n,P1", [(10**18, 1 << 22, 1600), (10**15, 10**6, 1024), (10**12, 3 * 10**6, 709)])
+def test_maximum_in_the_blocks_is_the_same_every_time(gbm, lo, n, P1):
+    """Chunks finish in any order, and whether one has to look its maximum up
+    depends on it; the segments' maxima do not."""
+    with gbm.Context(device=0, base_limit=2 * 10**9 if lo > 10**16 else 1 << 26, seg_len=1 << 20, p1=P1, p2=0) as g:
+        g.set_config(cover_prefix=1)
+        want = g.verify_range(lo, lo + 2 * n, segs=True, hist_cap=300)
+        g.set_config(cover_prefix=0)
+        for _ in range(40):
+            got = g.verify_range(lo, lo + 2 * n, segs=True, hist_cap=300)
+            assert got["segs"] == want["segs"]
+            np.testing.assert_array_equal(got["hist"], want["hist"])
