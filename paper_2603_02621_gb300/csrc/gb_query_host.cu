@@ -71,6 +71,44 @@ int gb_query_batch(gb_ctx* ctx, const uint64_t* n, uint32_t count, uint32_t P, u
 }
 
 
+}  // extern "C"
+
+namespace {
+
+// A stretch [a, b) of the n of a partition call: the pairs i < 480 O of all its n
+// by residues mod 15 (O = 0: none), the rest by the plain kernel
+struct Stretch {
+    uint64_t a, b, O;
+    uint32_t ny() const { return (uint32_t)((O + 95) / 96 * 96); }
+    uint32_t nz() const { return (uint32_t)(ny() + 15 * (((b - 4) / 2 - (a - 2) / 2) / 480 + 1) + 17); }
+};
+
+// Sums over many words for more than two warps of n go by residues mod 15, a
+// sixty-fourth of the way to the next multiple of lo at a time (the i up to
+// the first n's half are common to all, the rest is left to the plain
+// kernel); a residue's n come in blocks of 32, so fewer than 96 n would
+// mostly fill them with none (about 64 is where the two meet).
+std::vector<Stretch> partition_stretches(uint64_t lo, uint64_t hi)
+{
+    std::vector<Stretch> out;
+    for (uint64_t a = lo; a < hi;) {
+        uint64_t b = hi, O = 0;
+        if (a < (1u << 20)) b = std::min<uint64_t>(hi, 1u << 20);       // short sums: the plain kernel
+        if (a >= (1u << 20) && (hi - a) / 2 >= 96) {
+            b = std::min(hi, a + std::max<uint64_t>(960, a / 64 / 2 * 2));
+            if (hi - b < 192) b = hi;
+            O = gb::part_stream_words((a - 2) / 2 / 2 + 1);
+        }
+        out.push_back(Stretch{a, b, O});
+        a = b;
+    }
+    return out;
+}
+
+}  // namespace
+
+extern "C" {
+
 int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts)
 {
     if (!ctx || (hi > lo && !counts)) return fail(GB_EINVAL, "NULL argument");
@@ -89,6 +127,20 @@ int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts)
     if ((rc = ctx->part_p.ensure(words * 4)) || (rc = ctx->part_rev.ensure((words + 1) * 4)) ||
         (!out_dev && (rc = ctx->part_out.ensure(count * 4))))
         return rc;
+    // the residues' merged words, sized once for the stretch that needs most; without
+    // memory for them the plain kernel does the whole call
+    std::vector<Stretch> stretches = partition_stretches(lo, hi);
+    uint64_t ny = 0, nz = 0;
+    for (const Stretch& t : stretches)
+        if (t.O) {
+            ny = std::max<uint64_t>(ny, t.ny());
+            nz = std::max<uint64_t>(nz, t.nz());
+        }
+    if (ctx->part_y.ensure(32 * ny) || ctx->part_z.ensure(32 * nz)) {
+        ctx->part_y.release();
+        ctx->part_z.release();
+        stretches.assign(1, Stretch{lo, hi, 0});
+    }
     if ((rc = run_sieve(ctx, 1, words * 32, ctx->part_p.as<uint32_t>(), nullptr))) return rc;
     GB_LAUNCH(gb::launch_reverse_bits(ctx->part_p.as<uint32_t>(), ctx->part_rev.as<uint32_t>(), words, s));
     uint32_t* d_out = out_dev ? counts : ctx->part_out.as<uint32_t>();
@@ -98,48 +150,31 @@ int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts)
     pa.rev = ctx->part_rev.as<uint32_t>();
     pa.words = words;
     pa.run_words = 4096;
-    // Sums over many words for more than two warps of n go by residues mod 15, a
-    // sixty-fourth of the way to the next multiple of lo at a time (the i up to
-    // the first n's half are common to all, the rest is left to the plain
-    // kernel); a residue's n come in blocks of 32, so fewer than 96 n would
-    // mostly fill them with none (about 64 is where the two meet).
-    for (uint64_t a = lo; a < hi;) {
-        const uint64_t m_min = (a - 2) / 2;
-        uint64_t b = hi;
-        uint64_t O = 0;
-        if (a < (1u << 20)) b = std::min<uint64_t>(hi, 1u << 20);       // short sums: the plain kernel
-        if (a >= (1u << 20) && (hi - a) / 2 >= 96) {
-            b = std::min(hi, a + std::max<uint64_t>(960, a / 64 / 2 * 2));
-            if (hi - b < 192) b = hi;
-            O = gb::part_stream_words(m_min / 2 + 1);
-        }
-        if (O) {
+    for (const Stretch& t : stretches) {
+        if (t.O) {
             gb::PartCorrArgs ca{};
             ca.P = pa.P;
-            ca.m_min = m_min;
-            ca.m_max = (b - 4) / 2;
-            ca.O = (uint32_t)O;
-            ca.ny = (uint32_t)((O + 95) / 96 * 96);
-            const uint64_t blocks = (ca.m_max - m_min) / 480 + 1;
-            ca.nz = (uint32_t)(ca.ny + 15 * blocks + 17);
+            ca.m_min = (t.a - 2) / 2;
+            ca.m_max = (t.b - 4) / 2;
+            ca.O = (uint32_t)t.O;
+            ca.ny = t.ny();
+            ca.nz = t.nz();
             ca.run_words = 96 * 16;
-            if ((rc = ctx->part_y.ensure(32ull * ca.ny)) || (rc = ctx->part_z.ensure(32ull * ca.nz))) return rc;
             ca.y = ctx->part_y.as<uint32_t>();
             ca.z = ctx->part_z.as<uint32_t>();
-            ca.counts = d_out + (a - lo) / 2;
+            ca.counts = d_out + (t.a - lo) / 2;
             GB_LAUNCH(gb::launch_part_corr(ca, s));
             ctx->kernels += 1;                                          // (two kernels)
         }
-        pa.lo = a;
-        pa.count = (b - a) / 2;
+        pa.lo = t.a;
+        pa.count = (t.b - t.a) / 2;
         pa.n_blocks = (pa.count + 31) / 32;
-        pa.counts = d_out + (a - lo) / 2;
-        pa.w_first = 15 * O;
-        pa.with_3_5 = O != 0;
-        const uint64_t need = ((b - 4) / 2) / 2 / 32 + 1 - pa.w_first;  // words of the largest n
+        pa.counts = d_out + (t.a - lo) / 2;
+        pa.w_first = 15 * t.O;
+        pa.with_3_5 = t.O != 0;
+        const uint64_t need = ((t.b - 4) / 2) / 2 / 32 + 1 - pa.w_first;    // words of the largest n
         pa.runs = std::max<uint64_t>(1, (need + pa.run_words - 1) / pa.run_words);
         GB_LAUNCH(gb::launch_partitions(pa, s));
-        a = b;
     }
     if (!out_dev) GB_CUDA(ctx->copy(counts, d_out, count * 4, cudaMemcpyDeviceToHost, s));
     GB_CUDA(cudaStreamSynchronize(s));
