@@ -88,6 +88,11 @@ struct Stretch {
 // the first n's half are common to all, the rest is left to the plain
 // kernel); a residue's n come in blocks of 32, so fewer than 96 n would
 // mostly fill them with none (about 64 is where the two meet).
+// A stretch is three launches, some 60 us together where the sums are short: there
+// it takes 2^17 n, at most an eighth of the way.  2*10^5 n from 2^20 and from 2^21 on:
+// 0.47 and 0.63 ms; 1.43 and 1.28 by sixty-fourths, 1.20 and 2.03 by the plain
+// kernel (2*10^6 from 2^20: 6.6, 12.2, 24.9; stretches of 2^16 n 7.4, of 2^19 6.4; from
+// 2^24 on the sixty-fourth is as long).
 std::vector<Stretch> partition_stretches(uint64_t lo, uint64_t hi)
 {
     std::vector<Stretch> out;
@@ -95,7 +100,7 @@ std::vector<Stretch> partition_stretches(uint64_t lo, uint64_t hi)
         uint64_t b = hi, O = 0;
         if (a < (1u << 20)) b = std::min<uint64_t>(hi, 1u << 20);       // short sums: the plain kernel
         if (a >= (1u << 20) && (hi - a) / 2 >= 96) {
-            b = std::min(hi, a + std::max<uint64_t>(960, a / 64 / 2 * 2));
+            b = std::min(hi, a + std::max<uint64_t>(a / 64 / 2 * 2, std::min<uint64_t>(a / 8 / 2 * 2, 1u << 18)));
             if (hi - b < 192) b = hi;
             O = gb::part_stream_words((a - 2) / 2 / 2 + 1);
         }
