@@ -536,8 +536,8 @@ struct PartitionArgs {
     uint64_t runs;              // word runs per n-block
     uint64_t run_words;         // words per run
     uint32_t* counts;           // [count], zeroed; r(n) added
-    uint64_t w_first;           // first word of the sums (those before are counted by k_part_corr)
-    int with_3_5;               // add the pairs of 3 and 5
+    uint64_t w_first;           // first word of the sums (those before are counted by k_part_corr, without the
+                                // pairs of 3 and 5, which are added here); 0: all
 };
 // Pairs i < 480 O of many n by residues mod 15 (gb_partitions.cu)
 struct PartCorrArgs {

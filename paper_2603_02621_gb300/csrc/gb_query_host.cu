@@ -176,7 +176,6 @@ int gb_partitions(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t* counts)
         pa.n_blocks = (pa.count + 31) / 32;
         pa.counts = d_out + (t.a - lo) / 2;
         pa.w_first = 15 * t.O;
-        pa.with_3_5 = t.O != 0;
         const uint64_t need = ((t.b - 4) / 2) / 2 / 32 + 1 - pa.w_first;    // words of the largest n
         pa.runs = std::max<uint64_t>(1, (need + pa.run_words - 1) / pa.run_words);
         GB_LAUNCH(gb::launch_partitions(pa, s));
