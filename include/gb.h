@@ -65,8 +65,8 @@ typedef struct gb_config {
                                multiple of 8192, <= 2^20; 0 = 2^18.  Short
                                windows are cut into shorter tiles; long ones
                                go through slabs of up to 13 * 2^17 odd numbers
-                               while tile_bits, cta_threads and bucket_split
-                               are the defaults */
+                               while tile_bits, cta_threads and the split that
+                               results from bucket_split are the defaults */
     uint32_t cta_threads;   /* threads per segment-sieve CTA: 128, 256 or
                                512; 0 = 256 */
     uint32_t bucket_split;  /* sieving primes >= this are struck by the

@@ -158,9 +158,12 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
     // included).
     const gb_config& c = ctx->cfg;
     const int64_t last_num = B + 2 * (int64_t)(nbits - 1);
-    const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 32 && c.tile_bits == (1u << 18) &&
-                      c.bucket_split == 0 && c.cta_threads == 256 && ctx->mid_limit == (1u << 20) &&
-                      ctx->warp_split == 512 && nbits >= 8ull * gb::kSlabBits * gb::device_sms();
+    const uint64_t root = last_num > 0 ? isqrt_u64((uint64_t)last_num) : 0;
+    const bool tiling = c.tile_bits == (1u << 18) && c.cta_threads == 256 &&
+                        ctx->split(root) == gb_ctx::default_split(c.tile_bits, root);
+    const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 32 && tiling &&
+                      ctx->mid_limit == (1u << 20) && ctx->warp_split == 512 &&
+                      nbits >= 8ull * gb::kSlabBits * gb::device_sms();
     if (slab) nsmall = std::min<uint64_t>(np, ctx->pi((1u << 20) - 1));
     const bool large = np > nsmall && out;
     if (np > nsmall && !out) return fail(GB_EINVAL, "internal: large primes need an output buffer");

@@ -314,11 +314,11 @@ struct gb_ctx {
     // a wheel below 2^16) than through the tile sieve (measured on 2^34 even
     // n near 5e11 with the wheels in place: 2^13 15.33 ms per step, 2^14
     // 15.43, 2^15 15.78)
-    uint32_t split(uint64_t r) const
+    static uint32_t default_split(uint32_t tile_bits, uint64_t r)
     {
-        if (cfg.bucket_split) return cfg.bucket_split;
-        return r >= (1u << 18) ? std::min<uint32_t>(1u << 13, cfg.tile_bits) : cfg.tile_bits;
+        return r >= (1u << 18) ? std::min<uint32_t>(1u << 13, tile_bits) : tile_bits;
     }
+    uint32_t split(uint64_t r) const { return cfg.bucket_split ? cfg.bucket_split : default_split(cfg.tile_bits, r); }
 };
 
 // context configuration defaults and checks (gb_init, gb_set_config)
