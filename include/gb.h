@@ -66,7 +66,8 @@ typedef struct gb_config {
                                windows are cut into shorter tiles; long ones
                                go through slabs of up to 13 * 2^17 odd numbers
                                while tile_bits, cta_threads and the split that
-                               results from bucket_split are the defaults */
+                               results from bucket_split are the defaults, or
+                               gb_autotune's from a sample of shorter windows */
     uint32_t cta_threads;   /* threads per segment-sieve CTA: 128, 256 or
                                512; 0 = 256 */
     uint32_t bucket_split;  /* sieving primes >= this are struck by the

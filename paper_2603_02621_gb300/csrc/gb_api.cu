@@ -159,11 +159,11 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
     const gb_config& c = ctx->cfg;
     const int64_t last_num = B + 2 * (int64_t)(nbits - 1);
     const uint64_t root = last_num > 0 ? isqrt_u64((uint64_t)last_num) : 0;
-    const bool tiling = c.tile_bits == (1u << 18) && c.cta_threads == 256 &&
-                        ctx->split(root) == gb_ctx::default_split(c.tile_bits, root);
+    const bool tiling = ctx->tuned_tiles || (c.tile_bits == (1u << 18) && c.cta_threads == 256 &&
+                                             ctx->split(root) == gb_ctx::default_split(c.tile_bits, root));
     const bool slab = out && last_num > 0 && (uint64_t)last_num >= 1ull << 32 && tiling &&
                       ctx->mid_limit == (1u << 20) && ctx->warp_split == 512 &&
-                      nbits >= 8ull * gb::kSlabBits * gb::device_sms();
+                      nbits >= gb::slab_min_bits();
     if (slab) nsmall = std::min<uint64_t>(np, ctx->pi((1u << 20) - 1));
     const bool large = np > nsmall && out;
     if (np > nsmall && !out) return fail(GB_EINVAL, "internal: large primes need an output buffer");
@@ -446,6 +446,9 @@ int ctx_sieve_noalloc(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out)
 {
     return run_sieve(ctx, B, nbits, out, nullptr, false);
 }
+bool ctx_tuned_tiles(const gb_ctx* ctx) { return ctx->tuned_tiles; }
+void ctx_set_tuned_tiles(gb_ctx* ctx, bool tuned) { ctx->tuned_tiles = tuned; }
+uint64_t slab_min_bits() { return 8ull * kSlabBits * device_sms(); }
 int set_error(int code, const char* msg) { return fail(code, msg); }
 }  // namespace gb
 
@@ -543,6 +546,7 @@ int gb_init_shared(gb_ctx** out, const gb_ctx* parent, void* stream)
     ctx->L = parent->L;
     ctx->base = parent->base;
     ctx->warp_split = parent->warp_split;
+    ctx->tuned_tiles = parent->tuned_tiles;
     ctx->generic_cover = parent->generic_cover;
     ctx->batch_graph = parent->batch_graph;
     ctx->large_chunk_bits = parent->large_chunk_bits;
@@ -592,6 +596,9 @@ int gb_set_config(gb_ctx* ctx, const gb_config* cfg)
     GB_CUDA(cudaSetDevice(ctx->cfg.device));
     if (ctx->stream) GB_CUDA(cudaStreamSynchronize(ctx->stream));
     else GB_CUDA(cudaDeviceSynchronize());
+    if (c.tile_bits != ctx->cfg.tile_bits || c.cta_threads != ctx->cfg.cta_threads ||
+        c.bucket_split != ctx->cfg.bucket_split)
+        ctx->tuned_tiles = false;                           // the caller's own
     ctx->cfg = c;
     if (!getenv("GB_WARP_SPLIT")) ctx->warp_split = (int)std::min<uint32_t>(512, c.tile_bits / 64);
     return GB_OK;

@@ -211,6 +211,7 @@ struct SlabArgs {
     uint32_t slab_bits;         // set by the launcher: the slabs' length, a multiple of 4096
 };
 cudaError_t launch_slab(const SlabArgs& a, cudaStream_t s);
+uint64_t slab_min_bits();       // odd numbers from which a window may go through slabs: eight rounds of them
 // Primes from the slice limit to sqrt(B) over a window of several chunks of
 // 2^chunk_log2 bits (gb_large.cu): each prime started once per window and
 // carried from chunk to chunk -- per-prime next-multiple words for the primes
@@ -588,6 +589,10 @@ struct CtxView {
 };
 int ctx_view(const gb_ctx* ctx, CtxView* v);
 uint64_t ctx_pi(const gb_ctx* ctx, uint64_t x);            // primes <= x (x <= L)
+// whether the context's tile settings are the autotuner's, found on windows that
+// are too short for slabs
+bool ctx_tuned_tiles(const gb_ctx* ctx);
+void ctx_set_tuned_tiles(gb_ctx* ctx, bool tuned);
 // segment sieve of the odd numbers B + 2i, i < nbits, into out (device
 // words), with no device allocation: the large primes take the kernels that
 // strike in place (never the bucket lists, which are sized on first use)

@@ -216,6 +216,8 @@ struct gb_ctx {
     cudaGraphExec_t bgraph = nullptr;
     uint64_t work_strikes = 0, work_iters = 0, work_large = 0;
     int warp_split = 0;               // sieving primes below this strike one warp each
+    bool tuned_tiles = false;         // tile_bits, cta_threads and bucket_split come from gb_autotune on windows too
+                                      // short for slabs: long ones keep to slabs
     bool generic_cover = false;       // force the generic cover kernel (GB_COVER=generic)
     uint64_t large_chunk_bits = 1ull << 28;   // large-prime strikes per L2-resident chunk of the window
 

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include "gb.h"
+#include "gb_internal.cuh"
 
 namespace {
 
@@ -51,11 +52,12 @@ int run_sample(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_t cou
 }
 
 // best-of-reps time of the sample under cfg; < 0 if the setting is rejected
-double time_setting(gb_ctx* ctx, const gb_config& cfg, const uint64_t* lo, const uint64_t* hi, uint32_t count,
-                    int mode, uint32_t reps, std::vector<gb_segment_result>& recs, Timer& t, int* err)
+template <class Set>
+double time_setting(gb_ctx* ctx, const Set& set, const gb_config& cfg, const uint64_t* lo, const uint64_t* hi,
+                    uint32_t count, int mode, uint32_t reps, std::vector<gb_segment_result>& recs, Timer& t, int* err)
 {
     *err = GB_OK;
-    if (gb_set_config(ctx, &cfg) != GB_OK) return -1.0;
+    if (set(cfg, false) != GB_OK) return -1.0;
     cudaStream_t s = static_cast<cudaStream_t>(cfg.stream);
     int rc = run_sample(ctx, lo, hi, count, mode, recs);   // warm-up, arenas
     if (rc) {
@@ -163,6 +165,21 @@ extern "C" int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, 
     int rc = gb_get_config(ctx, &best);
     if (rc) return rc;
     const gb_config start = best;
+    // Tile settings found on windows too short for slabs (a batch has none) say
+    // nothing about longer ones, and leave those there; settings that the search
+    // does not change are the caller's as before.
+    uint64_t longest = 0;
+    for (uint32_t i = 0; i < count; ++i) longest = std::max(longest, (hi[i] - lo[i]) / 2);
+    const bool no_slabs = mode == GB_TUNE_BATCH || std::min(longest, best.slab_bits) + std::max(best.p1, best.p2) / 2 <
+                                                       gb::slab_min_bits();
+    const bool was_tuned = gb::ctx_tuned_tiles(ctx);
+    auto set = [&](const gb_config& c, bool tuned) {
+        const int e = gb_set_config(ctx, &c);
+        const bool own = c.tile_bits == start.tile_bits && c.cta_threads == start.cta_threads &&
+                         c.bucket_split == start.bucket_split;
+        if (e == GB_OK) gb::ctx_set_tuned_tiles(ctx, own ? was_tuned : tuned && no_slabs);
+        return e;
+    };
     // a result for this GPU, mode, setting and sample in the cache file
     const char* cache = std::getenv("GB_TUNE_CACHE");
     std::string key;
@@ -170,7 +187,7 @@ extern "C" int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, 
         key = tune_key(best, mode, lo, hi, count);
         gb_config hitc = best;
         double ms = 0;
-        if (gb_tune_cache_lookup(cache, key.c_str(), &hitc, &ms) == GB_OK && gb_set_config(ctx, &hitc) == GB_OK) {
+        if (gb_tune_cache_lookup(cache, key.c_str(), &hitc, &ms) == GB_OK && set(hitc, true) == GB_OK) {
             if (out) *out = hitc;
             if (best_ms) *best_ms = ms;
             return GB_OK;
@@ -179,14 +196,11 @@ extern "C" int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, 
     std::vector<gb_segment_result> recs(mode == GB_TUNE_BATCH ? count : 0);
     Timer t;
     int err = GB_OK;
-    double best_t = time_setting(ctx, best, lo, hi, count, mode, reps, recs, t, &err);
+    double best_t = time_setting(ctx, set, best, lo, hi, count, mode, reps, recs, t, &err);
     if (best_t < 0) {
-        gb_set_config(ctx, &start);
+        set(start, false);
         return err ? err : GB_EINVAL;
     }
-
-    uint64_t longest = 0;
-    for (uint32_t i = 0; i < count; ++i) longest = std::max(longest, (hi[i] - lo[i]) / 2);
 
     // candidates of one parameter, given the best setting so far
     using Apply = std::function<bool(gb_config&, uint32_t)>;
@@ -238,9 +252,9 @@ extern "C" int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, 
             gb_config c = best;
             if (!p.apply(c, v)) continue;
             if (std::memcmp(&c, &best, sizeof c) == 0) continue;
-            const double ms = time_setting(ctx, c, lo, hi, count, mode, reps, recs, t, &err);
+            const double ms = time_setting(ctx, set, c, lo, hi, count, mode, reps, recs, t, &err);
             if (err && err != GB_EINVAL) {
-                gb_set_config(ctx, &start);
+                set(start, false);
                 return err;
             }
             if (ms >= 0 && ms < best_t) {
@@ -249,7 +263,7 @@ extern "C" int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, 
             }
         }
     }
-    rc = gb_set_config(ctx, &best);
+    rc = set(best, true);
     if (rc) return rc;
     if (!key.empty()) gb_tune_cache_store(cache, key.c_str(), &best, best_t);   // a cache that cannot be written is skipped
     if (out) *out = best;

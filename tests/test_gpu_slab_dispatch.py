@@ -72,3 +72,40 @@ def test_slabs_against_the_oracle(gbm, oracle, A, rounds):
     _against_oracle(oracle, q, A, nbits, at)
     last = q[nbits // 64:].cpu().numpy().view(np.uint8)
     assert not np.unpackbits(last, bitorder="little")[nbits % 64:].any()
+
+
+def test_tuned_on_short_windows(gbm, monkeypatch, tmp_path):
+    """Tile settings that the autotuner found on a batch, or on windows without
+    slabs, leave long windows on their slabs; the same settings given by the
+    caller do not, nor do those found on a long window."""
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("GB_TUNE_CACHE", str(path))
+    nbits = _long()
+    q = torch.zeros(nbits // 64, dtype=torch.int64, device="cuda")
+    short = [(10**9, 10**9 + 2000), (10**9 + 4000, 10**9 + 4600)]
+    with gbm.Context(device=0, base_limit=1 << 20, p1=1 << 13, p2=0) as g:
+        for mode, sample, slabs in ((gbm.GB_TUNE_BATCH, short, True), (gbm.GB_TUNE_PLAIN, short, True),
+                                    (gbm.GB_TUNE_PLAIN, [(A - 1, A - 1 + 2 * nbits)], False)):
+            g.set_config(tile_bits=1 << 18, bucket_split=0, cta_threads=256, p1=1 << 13, cover_prefix=0, seg_len=1 << 24)
+            path.write_text("")
+            g.autotune(sample, mode, reps=1)
+            # what a search may come up with
+            key = path.read_text().split("\t")[0]
+            gbm.gb_tune_cache_store(str(path), key, dict(tile_bits=1 << 16, bucket_split=1 << 14, p1=1 << 13,
+                                                         cover_prefix=144, seg_len=1 << 24, cta_threads=128), 1.0)
+            g.set_config(tile_bits=1 << 18, bucket_split=0, cta_threads=256, p1=1 << 13, cover_prefix=0, seg_len=1 << 24)
+            cfg, ms = g.autotune(sample, mode, reps=1)
+            assert ms == 1.0 and cfg["tile_bits"] == 1 << 16
+            assert (_slices(gbm, g, A, nbits, q) == 0) == slabs, mode
+            g.set_config(seg_len=1 << 22)                     # not a tile setting
+            assert (_slices(gbm, g, A, nbits, q) == 0) == slabs, mode
+            with g.share() as h:
+                assert (_slices(gbm, h, A, nbits, q) == 0) == slabs, mode
+            g.set_config(cta_threads=512)
+            assert _slices(gbm, g, A, nbits, q) > 0
+            # a search that keeps the caller's tile settings leaves them the caller's
+            gbm.gb_tune_cache_store(str(path), key, dict(tile_bits=1 << 16, bucket_split=1 << 14, p1=1 << 12,
+                                                         cover_prefix=144, seg_len=1 << 24, cta_threads=512), 1.0)
+            g.set_config(p1=1 << 13)
+            g.autotune(sample, mode, reps=1)
+            assert g.config()["p1"] == 1 << 12 and _slices(gbm, g, A, nbits, q) > 0
