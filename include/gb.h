@@ -185,11 +185,12 @@ int gb_autotune(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_t co
                 gb_config* out, double* best_ms);
 /* Autotune cache.  When the environment variable GB_TUNE_CACHE names a file,
  * gb_autotune first looks up the key "<GPU name>|<SM count>|<mode>|<count>|
- * <hash of the sample's bounds>|<base_limit>|<p2>|<slab_bits>" there: on a
- * hit it applies the stored setting without timing anything (best_ms is the
- * stored time); otherwise it searches and appends one line
- * "<key>\t<tile_bits> <bucket_split> <p1> <cover_prefix> <seg_len>
- * <cta_threads> <best ms>".  The last line of a key wins; damaged lines are
+ * <hash of the sample's bounds>|<base_limit>|<p2>|<slab_bits>|k<kernels>" there
+ * (kernels: a number that changes with the library's kernels, so that settings
+ * found with others are not used): on a hit it applies the stored setting
+ * without timing anything (best_ms is the stored time); otherwise it searches
+ * and appends one line "<key>\t<tile_bits> <bucket_split> <p1> <cover_prefix>
+ * <seg_len> <cta_threads> <best ms>".  The last line of a key wins; damaged lines are
  * skipped.  Host-only helpers over that file format: lookup returns GB_OK and
  * fills those fields of *cfg (the rest untouched), GB_ERANGE when the key is
  * absent or the file cannot be read; store appends (GB_EINVAL if the file

@@ -84,9 +84,15 @@ double time_setting(gb_ctx* ctx, const Set& set, const gb_config& cfg, const uin
     return best;
 }
 
+// The kernels that a cached setting was found with: to be raised by one whenever
+// the sieve's or the cover's kernels or the rules that choose them change, so that
+// settings found with earlier ones are searched anew (2: slabs, the cover by
+// classes mod 3; keys before had none).
+constexpr int kTuneKernels = 2;
+
 // key of a tuning result: the GPU (name and SM count), the mode, the
-// settings that are not tuned (base primes, P2, slab) and the sample itself
-// (count and an FNV-1a hash of its bounds)
+// settings that are not tuned (base primes, P2, slab), the sample itself
+// (count and an FNV-1a hash of its bounds) and the kernels
 std::string tune_key(const gb_config& c, int mode, const uint64_t* lo, const uint64_t* hi, uint32_t count)
 {
     cudaDeviceProp prop{};
@@ -109,9 +115,9 @@ std::string tune_key(const gb_config& c, int mode, const uint64_t* lo, const uin
     for (char& ch : name)
         if (ch == '|' || ch == '\t' || ch == '\n') ch = '_';
     char buf[512];
-    std::snprintf(buf, sizeof buf, "%s|%d|%d|%u|%016llx|%llu|%u|%llu", name.c_str(), prop.multiProcessorCount, mode,
+    std::snprintf(buf, sizeof buf, "%s|%d|%d|%u|%016llx|%llu|%u|%llu|k%d", name.c_str(), prop.multiProcessorCount, mode,
                   count, (unsigned long long)h, (unsigned long long)c.base_limit, c.p2,
-                  (unsigned long long)c.slab_bits);
+                  (unsigned long long)c.slab_bits, kTuneKernels);
     return buf;
 }
 
