@@ -345,7 +345,7 @@ int gb_verify_range_noalloc(gb_ctx* ctx, uint64_t lo, uint64_t hi, uint32_t P,
  * context's stream around every launch while profiling is enabled.  Kinds:
  * 0 segment sieve, tile part or slabs (units: q bits sieved), 1 cover (units: even n;
  * batched mode: q bits), 2 retry pass (units: even n of the slabs it ran on),
- * 3 reductions and the max-only pass (units: segments), 4 segment sieve,
+ * 3 reductions (units: segments), 4 segment sieve,
  * primes above the tile split (units: q bits).  gb_profile_enable resets the
  * counters.  enable: 0 off; 1 (or any other nonzero value) event times and
  * the kernels' work counters (gb_profile_work); GB_PROFILE_EVENTS event

@@ -59,10 +59,6 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
     if (w_end > a.n_words) w_end = a.n_words;
     if (w_begin >= w_end) return;                           // past the range's end in its last segment
 
-    // max-only mode: only segments that no other pass gave a maximum
-    if (a.max_only && a.maxkey_check[seg] != 0) return;
-    const bool full = !a.max_only;
-
     for (uint32_t k = threadIdx.x; k < a.K; k += NT) sd[k] = (a.H - a.primes[1 + k] - 1) >> 1;
     for (uint32_t k = threadIdx.x; k <= a.K; k += NT) shist[k] = 0;
     if (threadIdx.x == 0) smax = 0;
@@ -70,7 +66,7 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long best = 0;
-    uint32_t* const pmin = full ? a.pmin : nullptr;
+    uint32_t* const pmin = a.pmin;
 
     for (uint64_t wb = w_begin + 32 * warp; wb < w_end; wb += 32 * (NT / 32)) {
         const uint64_t w = wb + lane;
@@ -118,7 +114,7 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
             const uint32_t tot = __reduce_add_sync(0xffffffffu, c);
             if (lane == 0 && tot) atomicAdd(&shist[k + 1], tot);
         }
-        if (full && active && C != ~0ull) {
+        if (active && C != ~0ull) {
             bool queued = false;
             if (a.retry) {
                 const unsigned int slot = atomicAdd(a.retry_count, 1u);
@@ -135,7 +131,7 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
             const unsigned long long key = ((unsigned long long)last_pidx1 << 32) | (0xffffffffull - j);
             if (key > best) best = key;
         }
-        if (full && a.iters) {
+        if (a.iters) {
             // primes applied until the word filled (all K when it did not)
             uint32_t it = active ? (C == ~0ull ? (last_pidx1 > 1 ? last_pidx1 - 1 : 0) : a.K) : 0;
             const uint32_t tot = __reduce_add_sync(0xffffffffu, it);
@@ -150,9 +146,8 @@ __global__ void __launch_bounds__(NT) k_cover(const CoverArgs a)
     if (lane == 0 && mhi) atomicMax(&smax, ((unsigned long long)mhi << 32) | mlo);
     __syncthreads();
     uint32_t* hrow = a.hist + (uint64_t)seg * a.hist_stride;
-    if (full)
-        for (uint32_t k = threadIdx.x; k <= a.K; k += NT)
-            if (shist[k]) atomicAdd(&hrow[k], shist[k]);
+    for (uint32_t k = threadIdx.x; k <= a.K; k += NT)
+        if (shist[k]) atomicAdd(&hrow[k], shist[k]);
     if (threadIdx.x == 0 && smax) atomicMax(&a.maxkey[seg], smax);
 }
 

@@ -292,10 +292,6 @@ struct CoverArgs {
     int has_n4;                 // slab starts at n = 4 (p_min(4) = 2)
     unsigned long long* iters;  // optional: sum over words of the primes applied
                                 // until the word filled (work count)
-    // generic kernel only: "max only" mode recomputes the segment maximum of
-    // segments whose key in maxkey_check is still 0 and writes it to maxkey
-    int max_only;
-    const unsigned long long* maxkey_check;
     // block cover only (set by the launcher)
     uint32_t n_later[3];        // blocks after block 0, of each class
     uint32_t halo_words;        // words below a word's partner of p = 3 that the blocks read

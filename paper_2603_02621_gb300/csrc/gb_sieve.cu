@@ -188,7 +188,6 @@ cudaError_t launch_sieve(const SieveArgs& a, int threads, cudaStream_t s)
     switch (threads) {
     case 128: return launch_sieve_nt<128>(a, s);
     case 512: return launch_sieve_nt<512>(a, s);
-    case 1024: return launch_sieve_nt<1024>(a, s);
     default: return launch_sieve_nt<256>(a, s);
     }
 }
