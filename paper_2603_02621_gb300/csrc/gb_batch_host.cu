@@ -24,9 +24,14 @@ int gb_verify_batch(gb_ctx* ctx, const uint64_t* lo, const uint64_t* hi, uint32_
     GB_CUDA(cudaSetDevice(cfg.device));
     cudaStream_t s = ctx->stream;
 
-    uint64_t n_words = 0;
-    for (uint32_t i = 0; i < count; ++i) n_words += hi[i] > lo[i] ? ((hi[i] - lo[i]) / 2 + 31) / 32 : 0;
-    const uint32_t cw = gb::cover_chunk_words(n_words, false);   // block-cover CTA chunk (32-bit words)
+    // block-cover CTA chunk (32-bit words), no longer than the longest range
+    uint64_t n_words = 0, longest = 1;
+    for (uint32_t i = 0; i < count; ++i) {
+        const uint64_t w = hi[i] > lo[i] ? ((hi[i] - lo[i]) / 2 + 31) / 32 : 0;
+        n_words += w;
+        longest = std::max(longest, w);
+    }
+    const uint32_t cw = (uint32_t)std::min<uint64_t>(gb::cover_chunk_words(n_words, false), longest);
 
     // per-range windows and work items
     uint64_t qwords = 0, n_sieve = 0, n_cover = 0, hi_max = 0, last_max = 0;

@@ -86,10 +86,11 @@ constexpr uint32_t kProbeWords = 3;
 // too small to give every SM its chunks.
 constexpr int kCoverNT = 512, kFusedNT = 256;
 constexpr int kCoverCtas = 2;                               // per SM
-// Chunks of at most 96 merged words (segments of 2^11 .. 2^13) are one warp per
-// class: CTAs of 128, eight per SM.  2^24 n near 1e12, segments of 2^11, 2^12 and
-// 2^13: 72, 39 and 25 us (319, 166 and 98 with CTAs of 512 whose first warp took
-// the three classes one after the other).
+// Chunks of at most 96 merged words (segments of 2^11 .. 2^13, batches of ranges of
+// at most 9216 n) are one warp per class: CTAs of 128, eight per SM.  2^24 n near
+// 1e12, segments of 2^11, 2^12 and 2^13: 72, 39 and 25 us (319, 166 and 98 with CTAs
+// of 512 whose first warp took the three classes one after the other); a batch of
+// 1000 ranges of 1000 n near 1e9: 22 us (37).
 constexpr int kShortNT = 128;
 constexpr int kMaxWarps = kCoverNT / 32;
 constexpr uint32_t kShortStream = 96;
@@ -950,7 +951,7 @@ cudaError_t launch_seg_cover(const CoverArgs& a0, const SieveArgs& sv, int KA, u
 // persistent: CTAs take (range, chunk) items from the queue until it is empty;
 // row r of the histograms, keys and counts is range r
 template <int NT, int L0>
-__global__ void __launch_bounds__(NT, kCoverCtas) k_cover_items(const CoverItemsArgs a)
+__global__ void __launch_bounds__(NT, kCoverCtas * kCoverNT / NT) k_cover_items(const CoverItemsArgs a)
 {
     extern __shared__ uint32_t smem[];
     __shared__ CoverShared sh;
@@ -977,10 +978,9 @@ __global__ void __launch_bounds__(NT, kCoverCtas) k_cover_items(const CoverItems
     }
 }
 
-template <int L0>
-static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
+template <int NT, int L0>
+static cudaError_t launch_items_nt(const CoverItemsArgs& a, cudaStream_t s)
 {
-    constexpr int NT = kCoverNT;
     const size_t smem = CoverSmem{stream_words(a.base.cta_words), a.base.halo_words}.bytes(NT / 32);
     auto k = k_cover_items<NT, L0>;
     cudaError_t e = allow_shared(k, max_cover_bytes(NT, kRounds));
@@ -991,10 +991,17 @@ static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <int L0>
+static cudaError_t launch_items_l0(const CoverItemsArgs& a, cudaStream_t s)
+{
+    return stream_words(a.base.cta_words) <= kShortStream ? launch_items_nt<kShortNT, L0>(a, s)
+                                                          : launch_items_nt<kCoverNT, L0>(a, s);
+}
+
 cudaError_t launch_cover_items(const CoverItemsArgs& a0, int KA, cudaStream_t s)
 {
     CoverItemsArgs a = a0;
-    a.split = 3ull * a.n_items_host <= (uint64_t)kCoverCtas * device_sms() ? 3u : 1u;     // (as launch_l0)
+    a.split = 3ull * a.n_items_host <= (uint64_t)kCoverCtas * device_sms() ? 3u : 1u;     // (as launch_nt)
     switch (cover_schedule(a.base, KA, kCoverNT / 32)) {
     case 24: return launch_items_l0<24>(a, s);
     case 32: return launch_items_l0<32>(a, s);
