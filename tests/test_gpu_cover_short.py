@@ -75,3 +75,18 @@ def test_maximum_in_the_blocks_is_the_same_every_time(gbm, lo, n, P1):
             got = g.verify_range(lo, lo + 2 * n, segs=True, hist_cap=300)
             assert got["segs"] == want["segs"]
             np.testing.assert_array_equal(got["hist"], want["hist"])
+
+
+def test_batches_of_short_ranges_time(gbm):
+    """1000 ranges of 1000 n: their cover in CTAs of 16 warps, the classes one
+    after the other, took 4.4 times as long as the generic cover of one of them,
+    in CTAs of 4 warps as long."""
+    ranges = [(10**9 + 40000 * i, 10**9 + 40000 * i + 2000) for i in range(1000)]
+    ms = []
+    with gbm.Context(device=0, base_limit=1 << 20, p1=1 << 15, p2=0) as g:
+        for _ in range(12):
+            gbm.gb_profile_enable(g.handle, gbm.GB_PROFILE_EVENTS)
+            g.verify_batch(ranges)
+            ms.append(gbm.gb_profile_read(g.handle)["cover"]["ms"])
+    one = _cover_ms(gbm, 10**9, 1000, p1=1 << 15, cover_prefix=1)
+    assert min(ms) < 2.2 * one, (min(ms), one)
