@@ -178,16 +178,19 @@ int run_sieve(gb_ctx* ctx, int64_t B, uint64_t nbits, uint32_t* out, unsigned lo
         sa.primes = a.primes;
         sa.recip = a.recip;
         sa.n_primes = (uint32_t)n;
-        // primes below 512 a warp each; without primes from 2^18 on, and so with
-        // little other work in a slab, below 1024 (2^32 odd numbers from 4 on: 1.47
-        // ms with 512, 1.35 with 1024, 1.44 with 1536; near 5e11, 2^33: 3.53, 3.70,
-        // 3.95).  The work counters keep to 512, as the tiles.
+        // primes below 512 a warp each and the wheel below 2^16 (as in the slices);
+        // without primes from 2^18 on, and so with little other work in a slab, below
+        // 1024 and below 2^18 (as in the tiles).  Nine rounds of slabs up to 2^33, 2^35,
+        // 2^36, 2^36.5, 2^37 and 2^39: 807, 850, 870, 885, 898 and 967 us with the first,
+        // 757, 802, 855, 891, 915 and 1050 with the second.  (A warp each below 1536 is
+        // slower than below 1024: 2^32 odd numbers from 4 on 1.44 and 1.35 ms.)  The work
+        // counters keep to 512, as the tiles.
         const bool low = last_num < 1ll << 36;
         const uint64_t nw = ctx->pi((low && !a.strikes ? 1024u : 512u) - 1);
         sa.n_warp = (uint32_t)std::min<uint64_t>(n, nw > first ? nw - first : 0);
         const uint64_t q = ctx->pi((1u << 13) - 1);
         sa.n_quad = (uint32_t)std::min<uint64_t>(n, std::max<uint64_t>(sa.n_warp, q > first ? q - first : 0));
-        sa.wheel_below = low ? 1u << 18 : 1u << 16;       // (as in the tiles; as in the slices)
+        sa.wheel_below = low ? 1u << 18 : 1u << 16;
         const uint64_t wb = ctx->pi(sa.wheel_below - 1);
         sa.n_plain = (uint32_t)std::min<uint64_t>(n, wb > first ? wb - first : 0);
         const uint64_t pm = n ? ctx->base->h_primes[nsmall - 1] : 0;

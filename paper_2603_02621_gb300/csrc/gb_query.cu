@@ -16,9 +16,10 @@
 // Bound: a query alone is a chain of two modular powers, base 2 and then the
 // eleven others side by side (before: twelve in sequence, in one thread); a
 // batch is bound by issue slots, of which the two powers take most.  On a
-// GB300, n uniform below 4e18: one query through gb_query 215.8 -> 62.3 us, a
-// batch of 4096 from host memory 1810 -> 136 us (one CTA of 128 threads per
-// query, every survivor tested to all twelve bases by its own thread, before).
+// GB300, n uniform below 4e18, the calls timed from Python, both kernels in turn on
+// one box: one query 197 to 274 us (with the n) -> 53 to 56, a batch of 4096 from
+// host memory 1786 -> 135 us (one CTA of 128 threads per query, every survivor
+// tested to all twelve bases by its own thread, before).
 #include "gb_internal.cuh"
 
 namespace gb {
