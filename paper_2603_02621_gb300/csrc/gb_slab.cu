@@ -335,11 +335,8 @@ __global__ void __launch_bounds__(kNT, 1) k_slab(const SlabArgs a)
                 if (p[u] < a.wheel_below) {
                     // only m p with m coprime to 30 (the stamp cleared the multiples
                     // of 3 and 5): see kHalfGaps30
-                    const uint32_t pm = p[u] % 30u;
-                    const uint32_t inv = pm * pm % 30u * pm % 30u;                  // p^-1 mod 30
-                    const uint32_t jr = (bmod30 + 2u * (i % 15u)) % 30u * inv % 30u >> 1;
-                    i += p[u] * ((kNextHalf30 >> (2 * jr)) & 3u);                   // < 2^21 + 4 * 2^20
-                    uint32_t g = __funnelshift_r(kHalfGaps30, kHalfGaps30, 4 * ((uint32_t)(kNextPos30 >> (3 * jr)) & 7u));
+                    uint32_t g;
+                    i += p[u] * wheel30_entry(p[u], bmod30, i % 15u, g);            // < 2^21 + 4 * 2^20
                     // four at a time: three consecutive half gaps sum to 7 at most
                     while (i + 7 * p[u] < nb) {
                         const uint32_t i1 = i + p[u] * (g & 15u), i2 = i1 + p[u] * ((g >> 4) & 15u),
