@@ -231,7 +231,9 @@ __global__ void __launch_bounds__(256) k_large(const LargeArgs a)
         uint32_t g = 0x11111111u;                           // half gaps: every odd multiple
         if (p < kMidWheelBelow) {
             // only m p with m coprime to 30 (see kHalfGaps30)
-            i += (uint64_t)p * wheel30_entry(p, pmod_u32(b, 30), (uint32_t)(i % 15u), g);
+            const uint32_t j = wheel30_at(p, pmod_u32(b, 30), (uint32_t)(i % 15u));
+            i += (uint64_t)p * wheel30_skip(j);
+            g = wheel30_gaps(j);
         }
         for (; i < span; g = __funnelshift_r(g, g, 4)) {
             const uint64_t bit = bit_lo + i;
@@ -357,8 +359,14 @@ __device__ __forceinline__ void mid_slice(int64_t B, uint64_t nbits, uint32_t* w
                 // the mod-30 wheel of the tile sieve (only m p with m coprime to
                 // 15), for primes with enough strikes per slice to pay for its start
                 if (j < nb) {
-                    uint32_t g;
-                    j += p[u] * wheel30_entry(p[u], bmod30, j % 15u, g);          // j + 3p < 2^22
+                    // (wheel30_at, _skip and _gaps written out: by the functions the slices of
+                    // 2^30 odd numbers near 1e13 take 279 us, so 275)
+                    const uint32_t pm = p[u] % 30u;
+                    const uint32_t inv = pm * pm % 30u * pm % 30u;                  // p^-1 mod 30
+                    const uint32_t jr = (bmod30 + 2u * (j % 15u)) % 30u * inv % 30u >> 1;
+                    const uint32_t pos = (uint32_t)(kNextPos30 >> (3 * jr)) & 7u;
+                    j += p[u] * ((kNextHalf30 >> (2 * jr)) & 3u);                 // j + 3p < 2^22
+                    uint32_t g = __funnelshift_r(kHalfGaps30, kHalfGaps30, 4 * pos);
                     for (; j < nb; g = __funnelshift_r(g, g, 4)) {
                         if (GB_DCHECK(j < kMidSliceBits, kDbgMidStrike))
                             atomicAnd(slice + (j >> 5), __funnelshift_l(0xfffffffeu, 0xfffffffeu, j));

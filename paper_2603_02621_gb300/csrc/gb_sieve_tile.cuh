@@ -47,17 +47,21 @@ constexpr uint32_t kHalfGaps30 = 0x13212123u;
 constexpr uint64_t kNextPos30 = 0x1ffdac8d2248ull;
 constexpr uint32_t kNextHalf30 = 0x6104118u;
 
-// The multiple b + 2 i of p (odd, i.e. m = (b + 2 i) / p odd), from b mod 30: how
-// many times p further on (in i) the first m coprime to 30 lies, and in `gaps` the
-// half gaps from there on, the next in the lowest 4 bits.  m = (b + 2 i) p^-1 with
-// p^-1 = p^3 (mod 30) (the units mod 30 have exponent 4).
-__device__ __forceinline__ uint32_t wheel30_entry(uint32_t p, uint32_t b_mod30, uint32_t i_mod15, uint32_t& gaps)
+// For the multiple b + 2 i of p (odd, i.e. m = (b + 2 i) / p odd), from b mod 30:
+// j, half the residue of m mod 30.  m = (b + 2 i) p^-1 with p^-1 = p^3 (mod 30)
+// (the units mod 30 have exponent 4).
+__device__ __forceinline__ uint32_t wheel30_at(uint32_t p, uint32_t b_mod30, uint32_t i_mod15)
 {
     const uint32_t pm = p % 30u;
     const uint32_t inv = pm * pm % 30u * pm % 30u;
-    const uint32_t j = (b_mod30 + 2u * i_mod15) % 30u * inv % 30u >> 1;
-    gaps = __funnelshift_r(kHalfGaps30, kHalfGaps30, 4 * ((uint32_t)(kNextPos30 >> (3 * j)) & 7u));
-    return (kNextHalf30 >> (2 * j)) & 3u;
+    return (b_mod30 + 2u * i_mod15) % 30u * inv % 30u >> 1;
+}
+// how many times p further on (in i) the first m coprime to 30 lies, and the half
+// gaps from there on, the next in the lowest 4 bits
+__device__ __forceinline__ uint32_t wheel30_skip(uint32_t j) { return (kNextHalf30 >> (2 * j)) & 3u; }
+__device__ __forceinline__ uint32_t wheel30_gaps(uint32_t j)
+{
+    return __funnelshift_r(kHalfGaps30, kHalfGaps30, 4 * ((uint32_t)(kNextPos30 >> (3 * j)) & 7u));
 }
 
 // one stamp table read at pattern offset a (a < period): 32 bits from bit a
@@ -224,8 +228,9 @@ __device__ __forceinline__ void sieve_tile(const SieveArgs& a, uint64_t t0, cons
             uint32_t i = s[u];
             if (p[u] < (1u << 20)) {
                 if (i < nb) {
-                    uint32_t g;
-                    i += p[u] * wheel30_entry(p[u], bmod30, i % 15u, g);     // i + 3p < 2^22: no wrap
+                    const uint32_t j = wheel30_at(p[u], bmod30, i % 15u);
+                    i += p[u] * wheel30_skip(j);                     // i + 3p < 2^22: no wrap
+                    uint32_t g = wheel30_gaps(j);
                     if (a.strikes) {
                         for (; i < nb; g = __funnelshift_r(g, g, 4)) {
                             strike(sm, i, a.tile_bits);

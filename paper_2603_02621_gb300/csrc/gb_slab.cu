@@ -335,8 +335,9 @@ __global__ void __launch_bounds__(kNT, 1) k_slab(const SlabArgs a)
                 if (p[u] < a.wheel_below) {
                     // only m p with m coprime to 30 (the stamp cleared the multiples
                     // of 3 and 5): see kHalfGaps30
-                    uint32_t g;
-                    i += p[u] * wheel30_entry(p[u], bmod30, i % 15u, g);            // < 2^21 + 4 * 2^20
+                    const uint32_t jr = wheel30_at(p[u], bmod30, i % 15u);
+                    i += p[u] * wheel30_skip(jr);                                   // < 2^21 + 4 * 2^20
+                    uint32_t g = wheel30_gaps(jr);
                     // four at a time: three consecutive half gaps sum to 7 at most
                     while (i + 7 * p[u] < nb) {
                         const uint32_t i1 = i + p[u] * (g & 15u), i2 = i1 + p[u] * ((g >> 4) & 15u),
